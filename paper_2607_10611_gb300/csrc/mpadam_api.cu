@@ -114,7 +114,31 @@ void make_scalars(const mpadam_config& c, int64_t t, StepScalars* s) {
   s->wmax = s->wmax_on ? c.w_max : 0.0f;
   s->wd_on = c.wd_add != 0.0f ? 1 : 0;
   s->kwd = static_cast<float>(static_cast<double>(c.lr_add) * static_cast<double>(c.wd_add));
-  s->cert_ok = (c.eps >= 0x1p-28f && c.tau >= 0x1p-125f && s->c2 <= 0x1p14f && c.lr_mul <= 4.0f) ? 1 : 0;
+  s->cert_ok = (c.eps >= 0x1p-28f && c.eps <= 0x1p60f && c.tau >= 0x1p-125f && s->c2 <= 0x1p14f &&
+                c.lr_mul <= 4.0f) ? 1 : 0;
+}
+
+uint64_t twice(float x) {
+  uint32_t b;
+  std::memcpy(&b, &x, sizeof b);
+  return (uint64_t)b << 32 | b;
+}
+
+void make_pairs(const StepScalars& s, mpadam::StepPairs* p) {
+  p->b1 = twice(s.b1);
+  p->b2 = twice(s.b2);
+  p->omb1 = twice(s.omb1);
+  p->omb2 = twice(s.omb2);
+  p->ka = twice(s.ka);
+  p->c2 = twice(s.c2);
+  p->km = twice(s.km);
+  p->ln2 = twice(s.ln2);
+  p->eps = twice(s.eps);
+  // the certified bound (derived beside madam_cert_pair)
+  p->nc1 = twice(-0x1.4p-19f);   // 5 2^-21
+  p->nc2 = twice(-0x1.4p-22f);   // 1.25 2^-22
+  p->nc0 = twice(-0x1p-96f);
+  p->m1 = twice(-1.0f);
 }
 
 // Philox4x32-10 round keys: key + r * (0x9E3779B9, 0xBB67AE85), r = 0..9.
@@ -488,6 +512,7 @@ void fill_common(StepArgs& a, const mpadam_config& cfg, const Geometry& geo, int
 
 void fill_step(StepArgs& a, const mpadam_config& cfg, int64_t step) {
   make_scalars(cfg, step, &a.s);
+  make_pairs(a.s, &a.p);
   a.t_lo = (uint32_t)(uint64_t)step;
   a.t_hi = (uint32_t)((uint64_t)step >> 32);
   a.e_cur_slot = (int32_t)(step % 2);

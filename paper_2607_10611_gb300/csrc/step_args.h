@@ -97,7 +97,15 @@ struct StepScalars {
   float gmax, wmax;  // active when gmax_on / wmax_on
   float kwd;         // eta_a * lambda, active when wd_on
   int32_t gmax_on, wmax_on, wd_on;
-  int32_t cert_ok;   // eps >= 2^-28, tau >= 2^-125, c2 <= 2^14, eta_m <= 4: certified fast path allowed
+  int32_t cert_ok;   // 2^-28 <= eps <= 2^60, tau >= 2^-125, c2 <= 2^14, eta_m <= 4: certified fast path allowed
+};
+
+// The scalars of the certified path's packed operations, twice each: the two
+// halves of an f32x2 operand.
+struct StepPairs {
+  uint64_t b1, b2, omb1, omb2, ka, c2, km, ln2, eps;
+  uint64_t nc1, nc2, nc0;  // minus the error bound's coefficients
+  uint64_t m1;             // -1
 };
 
 // A run of consecutive tiles of the tail pool.
@@ -121,6 +129,7 @@ struct StepArgs {
   int32_t off_g, off_m, off_v, off_ve;  // region offsets inside a stage (w at 0)
   int32_t off_s;             // block scales (kE4M3B, kNVFP4)
   StepScalars s;
+  StepPairs p;
   uint32_t rk0[kPhiloxRounds], rk1[kPhiloxRounds];  // Philox round keys: seed + r * Weyl
   uint32_t t_lo, t_hi;       // step number (Philox counter words 2, 3)
   // E4M3 delayed-scaling rings (caller-owned); unused for BF16 weights

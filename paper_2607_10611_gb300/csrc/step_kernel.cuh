@@ -239,97 +239,166 @@ __device__ __forceinline__ Upd madam_update(const StepScalars& s, float w, float
 }
 
 // ---------------------------------------------------------------------------
+// Packed binary32 pairs.  sm_103a multiplies and adds two binary32 values per
+// instruction (f32x2), each half rounded as the scalar operation is, so a
+// pair gives the same bits as two scalar operations with half the issue
+// slots.  The step's instances are bound by instruction issue before they
+// are by memory wherever an element has few bytes (BF16 moments, FP8 and FP4
+// weights).  With the packed update, the packed encoders and the tighter
+// bound below, instructions per element went from 84 to 61 (BF16 weights and
+// moments, SR) and from 115 to 83 (E4M3, SR); a 217 M-parameter list with BF16
+// moments went from 984 to 670 us (E4M3, nearest), 1135 to 880 (E4M3, SR),
+// 993 to 768 and 1085 to 911 (block-scaled E4M3), 867 to 804 and 1142 to 1048
+// (NVFP4); with binary32 moments NVFP4 with SR 1272 to 1225 us, E4M3 1152 to
+// 1099 (the others are bound by memory).
+// ---------------------------------------------------------------------------
+using f32x2 = uint64_t;  // low half: the even element
+
+__device__ __forceinline__ f32x2 pk(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpk(f32x2 x, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+}
+__device__ __forceinline__ f32x2 mul2_rn(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2_rd(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("mul.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2_ru(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2_rn(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2_rd(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2_ru(f32x2 x, f32x2 y) {
+  f32x2 r;
+  asm("add.rp.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2_rn(f32x2 x, f32x2 y, f32x2 z) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+  return r;
+}
+
+// ---------------------------------------------------------------------------
 // Certified fast update (Ziv's rounding test: A. Ziv, "Fast evaluation of
 // elementary mathematical functions with correctly rounded last bit", ACM
-// TOMS 17(3), 1991).  The moments are computed exactly as above; the two
-// square roots and three divisions of the weight update use the hardware
-// approximations sqrt.approx{.ftz}.f32 and div.approx{.ftz}.f32 (CUDA
-// documents at most 2 ulp for approximate division with divisors in
-// [2^-126, 2^126]).
-// With every approximate result assumed within 2^-19 relative of the
-// correctly rounded one -- 8x the documented bound -- plus an absolute 2^-126
-// for an operand or result flushed from the subnormal range, the fast weight
-// wn' differs from the canonical wn by at most
-//     eps = (|w u_m'| + |u_a'|) 2^-17 + (|w + w u_m'| + |wn'|) 2^-22 + 2^-96
-// (computed in the looser form (|w u_m'| + |u_a'|)(2^-17 + 2^-20)
-// + |w| 2^-21 (1 + 2^-20) + 2^-96, since |t| <= (|w| + |w u_m'|)(1 + 2^-24)
-// and |wn'| <= (|t| + |u_a'|)(1 + 2^-24))
-// (the relative errors propagate through the divisions, the clamp is
-// 1-Lipschitz, each of the two final roundings adds at most one ulp, and the
-// constants carry a further factor-of-two margin).  Flushing stays inside
-// the 2^-96 term and the relative terms when eps >= 2^-28, c2 <= 2^14 and
-// eta_m <= 4: a subnormal numerator of u_a or of n moves them by at most
-// 2^-126 / eps <= 2^-98 (and w u_m by at most eta_m 2^-98); a subnormal
-// nu or nu_e moves its denominator by at most c2 2^-63 <= 2^-21 eps; a
-// flushed u_m moves w u_m by at most |w| 2^-126.  The host enables this path
-// only under those conditions (cert_ok); divisors are checked in range here.  The caller stores the
-// encoding of wn' only when encoding wn' - eps (rounded down) and wn' + eps
-// (rounded up) gives the same code: every encoder here is monotone, so the
-// canonical wn, which lies in between, has that code too.  Otherwise the
-// element is recomputed with the exact sequence (madam_wn_exact).  Results
-// are therefore identical to the canonical sequence bit for bit; the test
-// only decides how much work that takes.
+// TOMS 17(3), 1991), two elements at a time.  The moments are computed
+// exactly as above; the weight update takes its two square roots from
+// sqrt.approx.ftz and its three quotients as products with rcp.approx.ftz
+// (the PTX manual bounds both by 2^-23 relative).
+//
+// With every approximate result assumed within 2^-21 relative of the exact
+// one and u = 2^-24 (one rounding):
+//   a denominator      fl(sqrt' c2 + eps): 2^-21 + 2u            = 1.25 2^-21
+//   u_a                + reciprocal 2^-21 + 2u                   = 2.5  2^-21
+//   n                  the same                                  = 2.5  2^-21
+//   w u_m              + 2u (eta_m n) + reciprocal 2^-21 + 2u    = 4    2^-21
+// (clamps are 1-Lipschitz and their intervals hold 0, so they keep relative
+// bounds), and the two last roundings, on either side, add
+// 2u (|t'| + |wn'|) <= 2u (2 |w| + 2 |w u_m'| + |u_a'|) with t = w + w u_m:
+//   eps = (|w u_m'| + |u_a'|) 5 2^-21 + rho 1.25 2^-22 + 2^-96
+// with rho = max(|w|, tau) >= |w|.  The constants leave a tenth to a quarter
+// for second-order terms and for the roundings of eps itself.  Flushing stays
+// inside these terms when eps >= 2^-28, c2 <= 2^14, eta_m <= 4 and tau >=
+// 2^-125: a subnormal nu or nu_e moves its denominator by at most
+// c2 2^-63 <= 2^-21 eps (in place of the square root's own 2^-21), a
+// subnormal numerator or quotient moves u_a and n by at most 2^-149 / eps <=
+// 2^-121 and w u_m by at most eta_m (|w| / rho) 2^-121.  A denominator is
+// infinite only when its moment is (eps <= 2^60, c2 <= 2^14), and then both
+// sides have a zero quotient.  The divisor rho needs no upper bound: above
+// 2^126 its approximate reciprocal is flushed to 0 and the canonical
+// |w u_m| <= eta_m |n| <= 4 (1 - beta2)^(-1/2) <= 2^14 (nu_e' >= (1 - beta2)
+// g_e^2 bounds |n|) is far below half an ulp of w, so w + w u_m is w on both
+// sides.  The host allows this path only under those conditions (cert_ok).
+// wn' not finite shows as a NaN in `fin` (the product with 0), and the group
+// is then recomputed.
+//
+// The caller stores the encoding of wn' only when encoding wn' - eps (rounded
+// down) and wn' + eps (rounded up) gives the same code: every encoder here is
+// monotone, so the canonical wn, which lies in between, has that code too.
+// Otherwise the element is recomputed with the exact sequence.  Results are
+// therefore identical to the canonical sequence bit for bit; the test only
+// decides how much work that takes.
 // ---------------------------------------------------------------------------
-// FTZ selects the flushing forms.  Both forms are covered by the same bound
-// (flushing is the larger error); every storage format uses the flushing
-// forms, which take fewer instructions (the non-flushing ones also handle
-// subnormal operands).
-template <bool FTZ>
-__device__ __forceinline__ float sqrt_approx(float x) {
+__device__ __forceinline__ float sqrt_approx_ftz(float x) {
   float y;
-  if (FTZ) asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  else asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-template <bool FTZ>
-__device__ __forceinline__ float div_approx(float a, float b) {
-  float q;
-  if (FTZ) asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
-  else asm("div.approx.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
-  return q;
+__device__ __forceinline__ float rcp_approx_ftz(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-struct CertUpd {
-  float wn, lo, hi;  // fast weight and the interval holding the canonical one
-  float e;           // the bound: lo = wn - e rounded down, hi = wn + e rounded up
-  float m, v, ve;    // exact moments
-  bool ok;           // divisors in the documented range and wn' finite
+struct CertPair {
+  f32x2 wn;  // fast weights
+  f32x2 ne;  // minus their bounds: the canonical weights lie in [wn + ne, wn - ne]
 };
 
-template <bool FTZ>
-__device__ __forceinline__ CertUpd madam_update_cert(const StepScalars& s, float w, float g, float m, float v,
-                                                     float ve) {
-  CertUpd o;
-  o.m = __fmaf_rn(s.b1, m, __fmul_rn(s.omb1, g));
-  o.v = __fmaf_rn(s.b2, v, __fmul_rn(s.omb2, __fmul_rn(g, g)));
-  const float ge = __fmul_rn(__fmul_rn(s.ln2, w), g);
-  o.ve = __fmaf_rn(s.b2, ve, __fmul_rn(s.omb2, __fmul_rn(ge, ge)));
-  const float den_a = __fmaf_rn(sqrt_approx<FTZ>(o.v), s.c2, s.eps);
-  const float ua = div_approx<FTZ>(__fmul_rn(s.ka, o.m), den_a);
-  const float den_e = __fmaf_rn(sqrt_approx<FTZ>(o.ve), s.c2, s.eps);
-  const float n = div_approx<FTZ>(ge, den_e);
-  const float rho = fmaxf(fabsf(w), s.tau);
-  float um = div_approx<FTZ>(__fmul_rn(s.km, n), rho);
-  um = fmaxf(s.lo, fminf(um, s.hi));
-  const float t = __fmaf_rn(w, um, w);
-  o.wn = __fadd_rn(t, ua);
-  // eps with (|t| + |wn'|) 2^-22 <= (2 |w| + 2 |w u_m'| + |u_a'|)(1 + 2^-23) 2^-22
-  // folded into the other two terms
-  const float e = __fmaf_rn(__fadd_rn(fabsf(__fmul_rn(w, um)), fabsf(ua)), 8.58306884765625e-06f /* 2^-17 + 2^-20 */,
-                            __fmaf_rn(fabsf(w), 4.768376129504759e-07f /* 2^-21 (1 + 2^-20) */,
-                                      1.2621774483536189e-29f /* 2^-96 */));
-  o.e = e;
-  o.lo = __fsub_rd(o.wn, e);
-  o.hi = __fadd_ru(o.wn, e);
-  // The two denominators must stay below 2^125 (their lower bound eps >=
-  // 2^-28 is checked on the host), and wn' must be finite.  The third divisor,
-  // rho = max(|w|, tau) >= tau >= 2^-125, needs no upper check: when |w| >
-  // 2^125 the canonical |w u_m| <= eta_m |n| <= 4 (1 - beta2)^(-1/2) <= 2^14
-  // (nu_e' >= (1 - beta2) g_e^2 bounds |n|; eta_m <= 4 on the host) is far
-  // below half an ulp of w, so w + w u_m rounds to w, as it does with the
-  // approximate quotient (documented within 2 ulp up to 2^126 and 0 above).
-  o.ok = fmaxf(den_a, den_e) <= 4.253529586511731e+37f /* 2^125 */ && fabsf(o.wn) < INFINITY;
+// m, v, ve go in as the stored moments and come back updated; `fin` collects
+// wn' 0 (NaN once any wn' is not finite).
+__device__ __forceinline__ CertPair madam_cert_pair(const StepScalars& s, const StepPairs& q, float w0, float w1,
+                                                    float g0, float g1, float& m0, float& m1, float& v0, float& v1,
+                                                    float& e0, float& e1, f32x2& fin) {
+  CertPair o;
+  const f32x2 w = pk(w0, w1), g = pk(g0, g1);
+  const f32x2 m = fma2_rn(q.b1, pk(m0, m1), mul2_rn(q.omb1, g));
+  const f32x2 v = fma2_rn(q.b2, pk(v0, v1), mul2_rn(q.omb2, mul2_rn(g, g)));
+  const f32x2 ge = mul2_rn(mul2_rn(q.ln2, w), g);
+  const f32x2 ve = fma2_rn(q.b2, pk(e0, e1), mul2_rn(q.omb2, mul2_rn(ge, ge)));
+  unpk(m, m0, m1);
+  unpk(v, v0, v1);
+  unpk(ve, e0, e1);
+  float d0, d1, x0, x1;
+  unpk(fma2_rn(pk(sqrt_approx_ftz(v0), sqrt_approx_ftz(v1)), q.c2, q.eps), d0, d1);
+  const f32x2 ua = mul2_rn(mul2_rn(q.ka, m), pk(rcp_approx_ftz(d0), rcp_approx_ftz(d1)));
+  unpk(fma2_rn(pk(sqrt_approx_ftz(e0), sqrt_approx_ftz(e1)), q.c2, q.eps), d0, d1);
+  const f32x2 n = mul2_rn(ge, pk(rcp_approx_ftz(d0), rcp_approx_ftz(d1)));
+  const float r0 = fmaxf(fabsf(w0), s.tau), r1 = fmaxf(fabsf(w1), s.tau);
+  unpk(mul2_rn(mul2_rn(q.km, n), pk(rcp_approx_ftz(r0), rcp_approx_ftz(r1))), x0, x1);
+  const f32x2 um = pk(fmaxf(s.lo, fminf(x0, s.hi)), fmaxf(s.lo, fminf(x1, s.hi)));
+  o.wn = add2_rn(fma2_rn(w, um, w), ua);
+  fin = fma2_rn(o.wn, 0ull, fin);
+  float a0, a1;
+  unpk(mul2_rn(w, um), x0, x1);
+  unpk(ua, a0, a1);
+  o.ne = fma2_rn(pk(__fadd_rn(fabsf(x0), fabsf(a0)), __fadd_rn(fabsf(x1), fabsf(a1))), q.nc1,
+                 fma2_rn(pk(r0, r1), q.nc2, q.nc0));
   return o;
+}
+
+// wn - ne rounded up (the product with -1 is exact).
+__device__ __forceinline__ f32x2 sub2_ru(f32x2 wn, f32x2 ne, const StepPairs& q) {
+  f32x2 r;
+  asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(ne), "l"(q.m1), "l"(wn));
+  return r;
+}
+
+// Whether any wn' collected in `fin` was not finite.
+__device__ __forceinline__ bool cert_not_finite(f32x2 fin) {
+  float a, b;
+  unpk(fin, a, b);
+  return !(a == 0.0f && b == 0.0f);
 }
 
 // The weight of the canonical sequence from the already updated (exact)
@@ -378,6 +447,13 @@ __device__ __forceinline__ float e4m3_value(uint32_t c) {
   return (c & 0x80u) ? -val : val;
 }
 
+// E2M1 code (sign, 2 exponent bits with bias 1, one mantissa bit) -> binary32 (exact).
+__device__ __forceinline__ float e2m1_value(uint32_t c) {
+  const uint32_t mag = c & 7u;
+  const uint32_t b = mag >= 2u ? ((((mag >> 1) + 126u) << 23) | ((mag & 1u) << 22)) : (mag ? 0x3F000000u : 0u);
+  return __uint_as_float(b | ((c & 8u) << 28));
+}
+
 // Eight E4M3 codes (bytes of r[0], r[1], lowest byte first) -> binary32.
 // E4M3 -> FP16 -> FP32 are both widening conversions, so this is exact
 // (NaN codes give NaN).
@@ -398,26 +474,72 @@ __device__ __forceinline__ void e4m3x8_to_f32(const uint32_t (&r)[2], float (&x)
   }
 }
 
-// Both ends of a bound interval (already scaled by 2^-e, outward rounded)
-// encoded at once in the E4M3 normal range: code of the lower end, and
-// whether the upper end has the same code.  Anything outside [2^-6, 448),
-// or a sign change, reports `same` = false (the caller then takes the exact
-// path, whose full encoder handles subnormals, saturation and NaN).
+// Eight bound intervals [lo, hi] (four pairs, already scaled by 2^-e, outward
+// rounded) -> packed E4M3 codes (element j in byte j of ow) and the mask of
+// undecided elements, whose bytes hold no code.  Magnitudes must stay below
+// 512 with both ends (the caller's amax or block scale sees to it).
+//
+// Nearest-even: the hardware conversion of both ends, two elements each.
+//
+// Stochastic: a normal E4M3 code is the binary32 magnitude's top 11 bits less
+// 960, one up iff r < (its low 20 bits) 2^12, i.e. iff the low 20 bits plus
+// 0xFFFFF - (r >> 12) carry.  Both ends add the same K - (r >> 12), K taking
+// off 960 + 9 as well, so their top 12 bits (sign, 11 bits of code - 9) are
+// the codes.  An element is undecided when those differ, or when its code -
+// 9 leaves [0, 128) (bits 27..30): subnormal codes, and code 8, which a
+// magnitude just below 2^-6 would round to on too fine a grid, go to the
+// exact encoder.  (Codes 127 and above are the caller's to rule out.)
 template <bool SR>
-__device__ __forceinline__ uint32_t e4m3_pair_normal(float xlo, float xhi, uint32_t r, bool& same) {
-  const uint32_t blo = __float_as_uint(xlo), bhi = __float_as_uint(xhi);
-  const uint32_t alo = blo & 0x7FFFFFFFu, ahi = bhi & 0x7FFFFFFFu;
-  uint32_t clo, chi;
-  if (SR) {
-    clo = (alo >> 20) + (r < (alo << 12) ? 1u : 0u);
-    chi = (ahi >> 20) + (r < (ahi << 12) ? 1u : 0u);
-  } else {  // nearest, ties to even: carry out of (rem + 0x7FFFF + lsb)
-    clo = (alo >> 20) + (((alo & 0xFFFFFu) + 0x7FFFFu + ((alo >> 20) & 1u)) >> 20);
-    chi = (ahi >> 20) + (((ahi & 0xFFFFFu) + 0x7FFFFu + ((ahi >> 20) & 1u)) >> 20);
+__device__ __forceinline__ uint32_t e4m3_interval_codes(const f32x2 (&lo)[4], const f32x2 (&hi)[4],
+                                                        const uint32_t (&rnd)[8], uint32_t (&ow)[2]) {
+  uint32_t mask = 0u;
+  if constexpr (SR) {
+    constexpr uint32_t K = 0xFFFFFu - (969u << 20);
+    uint32_t f[8], H[4], any = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float l0, l1, h0, h1;
+      unpk(lo[i], l0, l1);
+      unpk(hi[i], h0, h1);
+      const uint32_t q0 = K - (rnd[2 * i] >> 12), q1 = K - (rnd[2 * i + 1] >> 12);
+      const uint32_t s0 = __float_as_uint(l0) + q0, s1 = __float_as_uint(l1) + q1;
+      f[2 * i] = (s0 ^ (__float_as_uint(h0) + q0)) | (s0 & 0x78000000u);
+      f[2 * i + 1] = (s1 ^ (__float_as_uint(h1) + q1)) | (s1 & 0x78000000u);
+      any |= f[2 * i] | f[2 * i + 1];
+      H[i] = __byte_perm(s0, s1, 0x7632);  // sign | 4 bits | code - 9 | 4 bits, twice
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const uint32_t c = (__byte_perm(H[2 * i] >> 4, H[2 * i + 1] >> 4, 0x6420) & 0x7F7F7F7Fu) + 0x09090909u;
+      ow[i] = c ^ (__byte_perm(H[2 * i], H[2 * i + 1], 0x7531) & 0x80808080u);
+    }
+    if (any >> 20) {
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j)
+        if (f[j] >> 20) mask |= 1u << j;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      uint32_t cl, ch;
+      float l0, l1, l2, l3;
+      unpk(lo[2 * i], l0, l1);
+      unpk(lo[2 * i + 1], l2, l3);
+      asm("{\n .reg .b16 a, b;\n cvt.rn.satfinite.e4m3x2.f32 a, %2, %1;\n cvt.rn.satfinite.e4m3x2.f32 b, %4, %3;\n"
+          " mov.b32 %0, {a, b};\n}" : "=r"(cl) : "f"(l0), "f"(l1), "f"(l2), "f"(l3));
+      unpk(hi[2 * i], l0, l1);
+      unpk(hi[2 * i + 1], l2, l3);
+      asm("{\n .reg .b16 a, b;\n cvt.rn.satfinite.e4m3x2.f32 a, %2, %1;\n cvt.rn.satfinite.e4m3x2.f32 b, %4, %3;\n"
+          " mov.b32 %0, {a, b};\n}" : "=r"(ch) : "f"(l0), "f"(l1), "f"(l2), "f"(l3));
+      ow[i] = cl;
+      if (const uint32_t d = cl ^ ch) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((d >> (8 * j)) & 0xFFu) mask |= 1u << (4 * i + j);
+      }
+    }
   }
-  same = clo == chi && ((blo ^ bhi) >> 31) == 0u && (alo - 0x3C800000u) < (0x43E00000u - 0x3C800000u) &&
-         (ahi - 0x3C800000u) < (0x43E00000u - 0x3C800000u);
-  return ((blo >> 24) & 0x80u) | (clo - 960u);
+  return mask;
 }
 
 // binary32 (already scaled by 2^-e) -> E4M3 code, saturating at +-448.
@@ -721,13 +843,16 @@ __device__ __forceinline__ void group_random_bits(const StepArgs& a, uint64_t gi
 }
 
 // The canonical weight of slot j of consumer c (a runtime index), from the
-// original inputs in the stage at st (BF16 weights); the stage must still be
-// allocated.
-template <int GD, int MD>
-__device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, uint32_t st, int c, int j) {
+// original inputs in the stage at st, which must still be allocated.  dec:
+// the scale its code decodes with (E4M3 formats and NVFP4).
+template <int WD, int GD, int MD>
+__device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, uint32_t st, int c, int j, float dec) {
   constexpr int GS = esize_of(GD), MS = esize_of(MD);
   const uint32_t i = static_cast<uint32_t>(kGroup * c + j);
-  const float w = __uint_as_float(lds_u16(st + 2u * i) << 16);
+  float w;
+  if constexpr (WD == kBF16) w = __uint_as_float(lds_u16(st + 2u * i) << 16);
+  else if constexpr (WD == kNVFP4) w = __fmul_rn(e2m1_value((lds_u32(st + 4u * c) >> (4 * j)) & 0xFu), dec);
+  else w = __fmul_rn(e4m3_value(lds_u8(st + i)), dec);
   auto ld = [&](uint32_t base, int es) -> float {
     return es == 4 ? __uint_as_float(lds_u32(base + 4u * i)) : __uint_as_float(lds_u16(base + 2u * i) << 16);
   };
@@ -746,16 +871,26 @@ __device__ __forceinline__ uint32_t bf16_element_random_bits(const StepArgs& a, 
   return (j & 1) ? (~wd >> 16) : (~wd & 0xFFFFu);
 }
 
+// The 32-bit random lane of element j (a runtime index) of a group of E4M3 or
+// NVFP4 weights, as group_random_bits draws it.
+__device__ __forceinline__ uint32_t lane32_random_bits(const StepArgs& a, uint64_t gidx, int j) {
+  const uint64_t b = (gidx >> 2) + static_cast<uint64_t>(j >> 2);
+  const uint4 r = philox4x32_10(static_cast<uint32_t>(b), static_cast<uint32_t>(b >> 32), a.t_lo, a.t_hi, a.rk0,
+                                a.rk1);
+  const int q = j & 3;
+  return q == 0 ? r.x : (q == 1 ? r.y : (q == 2 ? r.z : r.w));
+}
+
 // Update 8 loaded elements and store them (vector stores when `vec` and
-// whole, else element by element).  STAGED (BF16 weights, whole staged
-// tiles): the stage at st stays allocated until this returns, and the
-// certified path's rare exact branch takes the undecided elements one at a
-// time from there (c: the consumer), in a loop over the set bits.  Otherwise
-// that branch uses the inputs held in registers.  (Measured on the 7B list:
-// keeping the inputs live through the certified loop for the exact branch,
-// 18.64 ms per step; this, 18.27 ms.  Reloading them from global memory was
-// slower still, 21.6 ms: about a tenth of the warps' groups take the branch,
-// and each reload waits on DRAM while the other warps wait for its stage.)
+// whole, else element by element).  STAGED (whole staged warps): the stage at
+// st stays allocated until this returns, and the certified path's rare exact
+// branch takes the undecided elements one at a time from there (c: the
+// consumer), in a loop over the set bits.  Otherwise that branch uses the
+// inputs held in registers.  (Measured on the 7B list: keeping the inputs
+// live through the certified loop for the exact branch, 18.64 ms per step;
+// this, 18.27 ms.  Reloading them from global memory was slower still, 21.6
+// ms: about a tenth of the warps' groups take the branch, and each reload
+// waits on DRAM while the other warps wait for its stage.)
 template <int WD, int GD, int MD, bool SR, bool OPT, bool STAGED>
 __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx& x, int64_t e0, int valid,
                                              float (&w)[8], float (&g)[8], float (&m)[8], float (&v)[8],
@@ -764,33 +899,35 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
   uint32_t rnd[8];
   if (SR) group_random_bits<WD>(a, static_cast<uint64_t>(x.d.goff + e0), rnd);
 
-  if (WD == kBF16 && !OPT && a.s.cert_ok) {  // certified fast path (see madam_update_cert)
-    uint32_t ow[4] = {0u, 0u, 0u, 0u};
-    uint32_t redo = 0u;
+  if (WD == kBF16 && !OPT && a.s.cert_ok) {  // certified fast path (see madam_cert_pair)
+    uint32_t ow[4], df[4];  // codes of the lower ends, and where the upper ends' differ (two 16-bit halves each)
+    f32x2 fin = 0ull;
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const CertUpd u = madam_update_cert<true>(a.s, w[j], g[j], m[j], v[j], ve[j]);
-      bool same;
-      uint32_t code;
+    for (int i = 0; i < 4; ++i) {
+      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+                                         m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
+      float l0, l1, h0, h1;
+      unpk(add2_rd(u.wn, u.ne), l0, l1);
+      unpk(sub2_ru(u.wn, u.ne, a.p), h0, h1);
       if (SR) {
-        const uint32_t slo = __float_as_uint(u.lo) + rnd[j], shi = __float_as_uint(u.hi) + rnd[j];
-        same = ((slo ^ shi) >> 16) == 0u;
-        code = slo >> 16;
+        ow[i] = __byte_perm(__float_as_uint(l0) + rnd[2 * i], __float_as_uint(l1) + rnd[2 * i + 1], 0x7632);
+        df[i] = ow[i] ^ __byte_perm(__float_as_uint(h0) + rnd[2 * i], __float_as_uint(h1) + rnd[2 * i + 1], 0x7632);
       } else {
-        const uint32_t pair = bf16x2_rn(u.lo, u.hi);
-        same = ((pair ^ (pair >> 16)) & 0xFFFFu) == 0u;
-        code = pair & 0xFFFFu;
+        ow[i] = bf16x2_rn(l0, l1);
+        df[i] = ow[i] ^ bf16x2_rn(h0, h1);
       }
-      ow[j >> 1] |= code << (16 * (j & 1));
-      if (!(u.ok && same)) redo |= 1u << j;
-      m[j] = u.m; v[j] = u.v; ve[j] = u.ve;
     }
-    if (redo) {  // rare: encode the canonical weight of the undecided elements
+    if ((df[0] | df[1] | df[2] | df[3]) != 0u || cert_not_finite(fin)) {
+      // rare: encode the canonical weight of the undecided elements
+      uint32_t redo = cert_not_finite(fin) ? 0xFFu : 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        redo |= ((df[i] & 0xFFFFu) ? 1u << (2 * i) : 0u) | ((df[i] >> 16) ? 2u << (2 * i) : 0u);
       if constexpr (STAGED) {
 #pragma unroll 1
         for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
           const int j = __ffs(rm) - 1;
-          const float xe = exact_wn_from_stage<GD, MD>(a, st, c, j);
+          const float xe = exact_wn_from_stage<WD, GD, MD>(a, st, c, j, 1.0f);
           const uint32_t code =
               SR ? (bf16_sr_sum(xe, bf16_element_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j)) >> 16)
                  : (bf16x2_rn(xe, xe) & 0xFFFFu);
@@ -815,35 +952,69 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
   } else if (WD == kE4M3 && !OPT && a.s.cert_ok) {
     // Certified fast path for E4M3: both ends of the bound are scaled by 2^-e
     // with outward rounding and encoded; the largest |w'| must be exact, so an
-    // element whose bound reaches the threshold is recomputed as well.  The
-    // threshold is the larger of this thread's running maximum and the
+    // element whose bound may reach the threshold is recomputed as well.  The
+    // threshold is the larger of this warp's running maximum and the
     // tensor's maximum flushed so far in this step: both are exact |w'| of
     // elements of this tensor, so no element below them can be the maximum.
-    uint32_t ow[2] = {0u, 0u};
-    uint32_t redo = 0u;
+    uint32_t ow[2];
     const float amax_f = fmaxf(__uint_as_float(amax_bits), x.amax_seed);
+    f32x2 fin = 0ull, lo[4], hi[4];
+    float top = 0.0f;  // the largest magnitude of any end
+    const f32x2 enc = pk(x.enc_scale, x.enc_scale);
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const CertUpd u = madam_update_cert<true>(a.s, w[j], g[j], m[j], v[j], ve[j]);
-      bool same;
-      const uint32_t code = e4m3_pair_normal<SR>(__fmul_rd(u.lo, x.enc_scale), __fmul_ru(u.hi, x.enc_scale),
-                                                 SR ? rnd[j] : 0u, same);
-      // an undecided element's code may be out of range (it is replaced
-      // below): keep it inside its own byte
-      ow[j >> 2] |= (code & 0xFFu) << (8 * (j & 3));
-      if (!(u.ok && same) || fmaxf(fabsf(u.lo), fabsf(u.hi)) >= amax_f) redo |= 1u << j;
-      m[j] = u.m; v[j] = u.v; ve[j] = u.ve;
+    for (int i = 0; i < 4; ++i) {
+      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+                                         m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
+      const f32x2 l = add2_rd(u.wn, u.ne), h = sub2_ru(u.wn, u.ne, a.p);
+      float l0, l1, h0, h1;
+      unpk(l, l0, l1);
+      unpk(h, h0, h1);
+      top = fmaxf(fmaxf(top, fabsf(l0)), fabsf(h0));
+      top = fmaxf(fmaxf(top, fabsf(l1)), fabsf(h1));
+      lo[i] = mul2_rd(l, enc);
+      hi[i] = mul2_ru(h, enc);
+    }
+    uint32_t redo = e4m3_interval_codes<SR>(lo, hi, rnd, ow);
+    const float sat = __fmul_rn(448.0f, x.cc_scale);  // 448 2^e: from here on codes saturate
+    if (top >= fminf(amax_f, sat) || cert_not_finite(fin)) {
+      if (!(top < sat) || cert_not_finite(fin)) {
+        redo = 0xFFu;
+      } else {
+        // maximum candidates: |w'| >= amax_f has a code at or above amax_f's own, rounded down
+        const float A = __fmul_rz(amax_f, x.enc_scale);
+        const uint32_t ab = __float_as_uint(A);
+        const uint32_t ca = ab >= 0x3C800000u ? (ab >> 20) - 960u : 0u;
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j)
+          if (((ow[j >> 2] >> (8 * (j & 3))) & 0x7Fu) >= ca) redo |= 1u << j;
+      }
     }
     if (redo) {  // rare: the canonical weight of undecided elements and maximum candidates
-#pragma unroll
-      for (int j = 0; j < kGroup; ++j) {
-        if ((redo >> j) & 1u) {
-          const float xe = madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
-          const uint32_t wb = __float_as_uint(xe) & 0x7FFFFFFFu;
-          if (j < valid && wb < 0x7F800000u) amax_bits = max(amax_bits, wb);
-          const uint32_t code = e4m3_encode<SR>(__fmul_rn(xe, x.enc_scale), SR ? rnd[j] : 0u);
+      auto exact_code = [&](int j, float xe, uint32_t r) {
+        const uint32_t wb = __float_as_uint(xe) & 0x7FFFFFFFu;
+        if (j < valid && wb < 0x7F800000u) amax_bits = max(amax_bits, wb);
+        return e4m3_encode<SR>(__fmul_rn(xe, x.enc_scale), r);
+      };
+      if constexpr (STAGED) {
+#pragma unroll 1
+        for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
+          const int j = __ffs(rm) - 1;
+          const uint32_t r = SR ? lane32_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j) : 0u;
+          const uint32_t code = exact_code(j, exact_wn_from_stage<WD, GD, MD>(a, st, c, j, x.dec_scale), r);
           const int sh = 8 * (j & 3);
-          ow[j >> 2] = (ow[j >> 2] & ~(0xFFu << sh)) | (code << sh);
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (i == (j >> 2)) ow[i] = (ow[i] & ~(0xFFu << sh)) | (code << sh);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) {
+          if ((redo >> j) & 1u) {
+            const uint32_t code =
+                exact_code(j, madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]), SR ? rnd[j] : 0u);
+            const int sh = 8 * (j & 3);
+            ow[j >> 2] = (ow[j >> 2] & ~(0xFFu << sh)) | (code << sh);
+          }
         }
       }
     }
@@ -944,78 +1115,104 @@ __device__ __forceinline__ uint32_t quad_max(uint32_t x) {
   return max(x, __shfl_xor_sync(0xFFFFFFFFu, x, 2));
 }
 
-template <int GD, int MD, bool SR, bool OPT>
+template <int GD, int MD, bool SR, bool OPT, bool STAGED>  // STAGED: see finish_group
 __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx& x, int64_t e0, int valid,
                                              uint32_t h_old, float (&w)[8], float (&g)[8], float (&m)[8],
-                                             float (&v)[8], float (&ve)[8]) {
+                                             float (&v)[8], float (&ve)[8], uint32_t st, int c) {
   uint32_t rnd[8];
-  if (SR) group_random_bits<kE4M3B>(a, static_cast<uint64_t>(x.d.goff + e0), rnd);
   const int32_t k_old = fp16_pow2_exponent(h_old);
   const uint32_t vmask = valid >= kGroup ? 0xFFu : (valid > 0 ? (1u << valid) - 1u : 0u);
-  uint32_t code[8];
+  uint32_t ow[2];
   int32_t k_new;
   if (!OPT && a.s.cert_ok) {
-    // Certified path (see madam_update_cert).  Keep the fast weights and the
+    // Certified path (see madam_cert_pair).  Keep the fast weights and the
     // thread's largest error bound et; the block maximum then lies in
     // [max |w'| - et, max |w'| + et] (outward rounded).  When both ends give
     // the same exponent (block_exponent is monotone) that is the exact one;
     // otherwise the quad computes its exact maximum.  Each element's code is
     // then taken from its interval [w' - et, w' + et] under the new scale
     // where both ends agree, else from the exact weight.
-    float wf[8];
-    float et = 0.0f, am = 0.0f;
-    uint32_t bad = 0u;
+    f32x2 wf[4], fin = 0ull;
+    float nt = 0.0f, am = 0.0f;  // nt = -et
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const CertUpd u = madam_update_cert<true>(a.s, w[j], g[j], m[j], v[j], ve[j]);
-      wf[j] = u.wn;
-      m[j] = u.m; v[j] = u.v; ve[j] = u.ve;
-      if (!u.ok) {
-        bad |= 1u << j;
+    for (int i = 0; i < 4; ++i) {
+      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+                                         m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
+      float x0, x1, n0, n1;
+      unpk(u.wn, x0, x1);
+      unpk(u.ne, n0, n1);
+      wf[i] = u.wn;
+      nt = fminf(fminf(nt, n0), n1);
+      if (valid >= kGroup) {
+        am = fmaxf(fmaxf(am, fabsf(x0)), fabsf(x1));
       } else {
-        et = fmaxf(et, u.e);
-        if ((vmask >> j) & 1u) am = fmaxf(am, fabsf(u.wn));
+        if ((vmask >> (2 * i)) & 1u) am = fmaxf(am, fabsf(x0));
+        if ((vmask >> (2 * i + 1)) & 1u) am = fmaxf(am, fabsf(x1));
       }
     }
-    bad &= vmask;
-    const float lo_t = bad ? 0.0f : fmaxf(__fsub_rd(am, et), 0.0f);
-    const float hi_t = bad ? INFINITY : __fadd_ru(am, et);
+    const bool bad = cert_not_finite(fin);
+    const float lo_t = bad ? 0.0f : fmaxf(__fadd_rd(am, nt), 0.0f);
+    const float hi_t = bad ? INFINITY : __fsub_ru(am, nt);
     const uint32_t qlo = quad_max(__float_as_uint(lo_t));  // non-negative floats order as their bits
     const uint32_t qhi = quad_max(__float_as_uint(hi_t));
     const int32_t kl = block_exponent(qlo, k_old);
     const bool certain = qlo != 0u && qhi < 0x7E800000u /* 2^126 */ && kl == block_exponent(qhi, k_old);
     k_new = kl;
+    auto exact_wn = [&](int j) -> float {
+      if constexpr (STAGED) return exact_wn_from_stage<kE4M3B, GD, MD>(a, st, c, j, fp16_value(h_old));
+      else return madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
+    };
     if (__any_sync(0xFFFFFFFFu, !certain)) {  // exact block maximum for the undecided quads
       uint32_t amx = 0u;
       if (!certain) {
-#pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
+        auto take = [&](int j) {
           if ((vmask >> j) & 1u) {
-            const uint32_t b = __float_as_uint(madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j])) & 0x7FFFFFFFu;
+            const uint32_t b = __float_as_uint(exact_wn(j)) & 0x7FFFFFFFu;
             if (b < 0x7F800000u) amx = max(amx, b);
           }
+        };
+        if constexpr (STAGED) {
+#pragma unroll 1
+          for (int j = 0; j < kGroup; ++j) take(j);
+        } else {
+#pragma unroll
+          for (int j = 0; j < kGroup; ++j) take(j);
         }
       }
       amx = quad_max(amx);
       if (!certain) k_new = block_exponent(amx, k_old);
     }
     const float enc = pow2f(-k_new);
-    uint32_t redo = bad;
+    const f32x2 enc2 = pk(enc, enc), nt2 = pk(nt, nt);
+    f32x2 lo[4], hi[4];
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      bool same;
-      code[j] = e4m3_pair_normal<SR>(__fmul_rd(__fsub_rd(wf[j], et), enc), __fmul_ru(__fadd_ru(wf[j], et), enc),
-                                     SR ? rnd[j] : 0u, same);
-      if (!same) redo |= 1u << j;
+    for (int i = 0; i < 4; ++i) {
+      lo[i] = mul2_rd(add2_rd(wf[i], nt2), enc2);
+      hi[i] = mul2_ru(sub2_ru(wf[i], nt2, a.p), enc2);
     }
+    if (SR) group_random_bits<kE4M3B>(a, static_cast<uint64_t>(x.d.goff + e0), rnd);
+    uint32_t redo = e4m3_interval_codes<SR>(lo, hi, rnd, ow);
+    // past the largest scale codes saturate (448 2^15); elsewhere the scale covers the block
+    if (bad || (k_new == 15 && qhi >= 0x4B600000u)) redo = 0xFFu;
     redo &= vmask;
     if (redo) {  // rare: the canonical weight of the undecided elements
+      auto put = [&](int j, uint32_t r) {
+        const uint32_t code = e4m3_encode<SR>(__fmul_rn(exact_wn(j), enc), r);
+        const int sh = 8 * (j & 3);
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) {
-        if ((redo >> j) & 1u) {
-          const float xe = madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
-          code[j] = e4m3_encode<SR>(__fmul_rn(xe, enc), SR ? rnd[j] : 0u);
+        for (int i = 0; i < 2; ++i)
+          if (i == (j >> 2)) ow[i] = (ow[i] & ~(0xFFu << sh)) | (code << sh);
+      };
+      if constexpr (STAGED) {
+#pragma unroll 1
+        for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
+          const int j = __ffs(rm) - 1;
+          put(j, SR ? lane32_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j) : 0u);
         }
+      } else {
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j)
+          if ((redo >> j) & 1u) put(j, SR ? rnd[j] : 0u);
       }
     }
   } else {
@@ -1030,12 +1227,12 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
     }
     k_new = block_exponent(quad_max(amx), k_old);
     const float enc = pow2f(-k_new);
+    if (SR) group_random_bits<kE4M3B>(a, static_cast<uint64_t>(x.d.goff + e0), rnd);
+    ow[0] = ow[1] = 0u;
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) code[j] = e4m3_encode<SR>(__fmul_rn(wn[j], enc), SR ? rnd[j] : 0u);
+    for (int j = 0; j < kGroup; ++j)
+      ow[j >> 2] |= e4m3_encode<SR>(__fmul_rn(wn[j], enc), SR ? rnd[j] : 0u) << (8 * (j & 3));
   }
-  uint32_t ow[2];
-  ow[0] = code[0] | (code[1] << 8) | (code[2] << 16) | (code[3] << 24);
-  ow[1] = code[4] | (code[5] << 8) | (code[6] << 16) | (code[7] << 24);
   put_e4m3(ow, x.d.w, e0, valid, x.vec);
   const uint32_t h_new = fp16_pow2_bits(k_new);
   if ((threadIdx.x & 3) == 0 && valid > 0) static_cast<uint16_t*>(x.scale)[e0 / kBlock] = static_cast<uint16_t>(h_new);
@@ -1080,7 +1277,7 @@ __device__ __forceinline__ void general_block_group(const StepArgs& a, const Ten
     get_bf16<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
     get_bf16<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
   }
-  finish_block<GD, MD, SR, OPT>(a, x, e0, valid, h, w, g, m, v, ve);
+  finish_block<GD, MD, SR, OPT, false>(a, x, e0, valid, h, w, g, m, v, ve, st, c);
 }
 
 // The same, as a call: with BF16 moments, as for general_group_call.  Inline,
@@ -1100,12 +1297,6 @@ __device__ __noinline__ void general_block_group_call(const StepArgs& a, const T
 // x = w' / d' (correctly rounded) under the block's new scale.  The two
 // threads of a pair (lanes 2p, 2p+1) hold one block.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float e2m1_value(uint32_t c) {
-  const uint32_t mag = c & 7u;
-  const uint32_t b = mag >= 2u ? ((((mag >> 1) + 126u) << 23) | ((mag & 1u) << 22)) : (mag ? 0x3F000000u : 0u);
-  return __uint_as_float(b | ((c & 8u) << 28));
-}
-
 // binary32 -> E2M1 code: nearest-even, or stochastic (away from zero iff
 // r < floor(fraction * 2^32)); |x| >= 6 and infinities saturate; NaN -> +0.
 // Branch-free: with the grid spacing sp = 0.5, 1 or 2 of |x|'s binade
@@ -1226,7 +1417,8 @@ __device__ __forceinline__ Fp4Code nvfp4_scale_code(float A, float G, uint32_t c
     r.p = __fmul_rn(6.0f, r.d);
     return r;
   }
-  const float est = div_approx<false>(A, __fmul_rn(6.0f, G));
+  float est;
+  asm("div.approx.f32 %0, %1, %2;" : "=f"(est) : "f"(A), "f"(__fmul_rn(6.0f, G)));
   int32_t c = static_cast<int32_t>(e4m3_encode<true>(est, 0u) & 0x7Fu);  // random bits 0: rounds up
   c = c < 1 ? 1 : (c > 126 ? 126 : c);
   const Fp4Code hi = fp4_code(static_cast<uint32_t>(c), G);
@@ -1254,25 +1446,6 @@ __device__ __forceinline__ void put_fp4(uint32_t packed, void* w, int64_t e0, in
 
 __device__ __forceinline__ uint32_t pair_max(uint32_t x) {
   return max(x, __shfl_xor_sync(0xFFFFFFFFu, x, 1));
-}
-
-// One element's canonical update recomputed from the stage's original
-// inputs (kept until the group is done): the exact weight of the element's
-// group slot j.
-template <int GD, int MD>
-__device__ __forceinline__ float fp4_exact_from_stage(const StepArgs& a, uint32_t st, int c, int j, float d_old) {
-  constexpr int GS = esize_of(GD), MS = esize_of(MD);
-  const uint32_t word = lds_u32(st + 4 * c);
-  float q[8];
-  e2m1x8_to_f32(word, q);
-  const float w = __fmul_rn(q[j], d_old);
-  auto ld = [&](uint32_t base, int es) -> float {
-    const uint32_t addr = base + static_cast<uint32_t>(kGroup * es * c + es * j);
-    return es == 4 ? __uint_as_float(lds_u32(addr)) : __uint_as_float(lds_u16(addr) << 16);
-  };
-  const float g = ld(st + a.off_g, GS);
-  const float m = ld(st + a.off_m, MS), v = ld(st + a.off_v, MS), ve = ld(st + a.off_ve, MS);
-  return madam_update<false>(a.s, w, g, m, v, ve).wn;
 }
 
 // One element's canonical weight recomputed from global memory after the
@@ -1323,7 +1496,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
   float d;
   static_assert(SRC != kExactGlobal || MD == kF32, "exact recompute from global needs binary32 moments");
   auto exact_wn = [&](int j) -> float {
-    if constexpr (SRC == kExactStage) return fp4_exact_from_stage<GD, MD>(a, st, c, j, d_old);
+    if constexpr (SRC == kExactStage) return exact_wn_from_stage<kNVFP4, GD, MD>(a, st, c, j, d_old);
     else if constexpr (SRC == kExactGlobal) return fp4_exact_from_global<GD>(a, x, e0 + j, d_old);
     else return madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
   };
@@ -1333,22 +1506,26 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
     // maximum where they do not); then each element's interval, divided by
     // d through an approximate reciprocal, is encoded at both ends.
     float wf[8];
-    float et = 0.0f, am = 0.0f;
-    uint32_t bad = 0u;
+    float nt = 0.0f, am = 0.0f;
+    f32x2 fin = 0ull;
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const CertUpd u = madam_update_cert<true>(a.s, w[j], g[j], m[j], v[j], ve[j]);
-      wf[j] = u.wn;
-      m[j] = u.m; v[j] = u.v; ve[j] = u.ve;
-      if (!u.ok) {
-        bad |= 1u << j;
+    for (int i = 0; i < 4; ++i) {
+      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+                                         m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
+      float n0, n1;
+      unpk(u.wn, wf[2 * i], wf[2 * i + 1]);
+      unpk(u.ne, n0, n1);
+      nt = fminf(fminf(nt, n0), n1);
+      if (valid >= kGroup) {
+        am = fmaxf(fmaxf(am, fabsf(wf[2 * i])), fabsf(wf[2 * i + 1]));
       } else {
-        et = fmaxf(et, u.e);
-        if ((vmask >> j) & 1u) am = fmaxf(am, fabsf(u.wn));
+        if ((vmask >> (2 * i)) & 1u) am = fmaxf(am, fabsf(wf[2 * i]));
+        if ((vmask >> (2 * i + 1)) & 1u) am = fmaxf(am, fabsf(wf[2 * i + 1]));
       }
     }
     if constexpr (SRC != kExactRegs) put_moments<MD, !SR>(x, e0, valid, m, v, ve);
-    bad &= vmask;
+    const float et = -nt;
+    const uint32_t bad = cert_not_finite(fin) ? vmask : 0u;
     const float lo_t = bad ? 0.0f : fmaxf(__fsub_rd(am, et), 0.0f);
     const float hi_t = bad ? INFINITY : __fadd_ru(am, et);
     const uint32_t plo = pair_max(__float_as_uint(lo_t));
@@ -1708,9 +1885,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     const int kt = stage_k[s];
     if (kt != k) {  // another tensor: flush this one's E4M3 amax
       if (WD == kE4M3 && k >= 0) {
-        const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
-        if (lane == 0 && wmax != 0u)
-          atomicMax(&a.fp8_amax[static_cast<int64_t>(a.a_next_slot) * n + x.d.ring], wmax);
+        if (lane == 0 && amax_bits != 0u)
+          atomicMax(&a.fp8_amax[static_cast<int64_t>(a.a_next_slot) * n + x.d.ring], amax_bits);
         amax_bits = 0u;
       }
       enter(kt);
@@ -1763,17 +1939,16 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         finish_fp4<GD, MD, SR, OPT, kExactStage>(a, x, e0, kGroup, h_old, w, g, m, v, ve, st, c);
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));
-      } else if constexpr (WD == kBF16) {
+      } else {
         // the stage stays until the group is done: the rare exact branch reads
         // its inputs there
-        finish_group<WD, GD, MD, SR, OPT, true>(a, x, e0, kGroup, w, g, m, v, ve, amax_bits, st, c);
+        if constexpr (WD == kE4M3B) finish_block<GD, MD, SR, OPT, true>(a, x, e0, kGroup, h_old, w, g, m, v, ve, st, c);
+        else finish_group<WD, GD, MD, SR, OPT, true>(a, x, e0, kGroup, w, g, m, v, ve, amax_bits, st, c);
         __syncwarp();
+        // one running maximum per warp: the lanes' own would each reach the
+        // threshold again and again, in nearly every tile of some lane
+        if (WD == kE4M3) amax_bits = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
         if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));
-      } else {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));
-        if constexpr (WD == kE4M3B) finish_block<GD, MD, SR, OPT>(a, x, e0, kGroup, h_old, w, g, m, v, ve);
-        else finish_group<WD, GD, MD, SR, OPT, false>(a, x, e0, kGroup, w, g, m, v, ve, amax_bits, st, c);
       }
       if (++s == S) { s = 0; ++use; }
       continue;
@@ -1796,13 +1971,12 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
                              : general_group_call<WD, GD, MD, SR, OPT>(
                                    a, x, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes), amax_bits);
     __syncwarp();
+    if (WD == kE4M3) amax_bits = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
     if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));
     if (++s == S) { s = 0; ++use; }
   }
-  if (WD == kE4M3 && k >= 0) {
-    const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
-    if (lane == 0 && wmax != 0u) atomicMax(&a.fp8_amax[static_cast<int64_t>(a.a_next_slot) * n + x.d.ring], wmax);
-  }
+  if (WD == kE4M3 && k >= 0 && lane == 0 && amax_bits != 0u)
+    atomicMax(&a.fp8_amax[static_cast<int64_t>(a.a_next_slot) * n + x.d.ring], amax_bits);
 }
 
 }  // namespace mpadam
