@@ -115,7 +115,7 @@ void make_scalars(const mpadam_config& c, int64_t t, StepScalars* s) {
   s->wd_on = c.wd_add != 0.0f ? 1 : 0;
   s->kwd = static_cast<float>(static_cast<double>(c.lr_add) * static_cast<double>(c.wd_add));
   s->cert_ok = (c.eps >= 0x1p-28f && c.eps <= 0x1p60f && c.tau >= 0x1p-125f && s->c2 <= 0x1p14f &&
-                c.lr_mul <= 4.0f) ? 1 : 0;
+                c.lr_mul <= 4.0f && s->kwd <= 1.0f) ? 1 : 0;
 }
 
 uint64_t twice(float x) {
@@ -134,9 +134,10 @@ void make_pairs(const StepScalars& s, mpadam::StepPairs* p) {
   p->km = twice(s.km);
   p->ln2 = twice(s.ln2);
   p->eps = twice(s.eps);
+  p->kwd = twice(s.kwd);
   // the certified bound (derived beside madam_cert_pair)
   p->nc1 = twice(-0x1.4p-19f);   // 5 2^-21
-  p->nc2 = twice(-0x1.4p-22f);   // 1.25 2^-22
+  p->nc2 = twice(s.wd_on ? -0x1.4p-21f : -0x1.4p-22f);  // 1.25 2^-22, twice with decay
   p->nc0 = twice(-0x1p-96f);
   p->m1 = twice(-1.0f);
 }

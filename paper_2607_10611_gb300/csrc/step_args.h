@@ -97,13 +97,13 @@ struct StepScalars {
   float gmax, wmax;  // active when gmax_on / wmax_on
   float kwd;         // eta_a * lambda, active when wd_on
   int32_t gmax_on, wmax_on, wd_on;
-  int32_t cert_ok;   // 2^-28 <= eps <= 2^60, tau >= 2^-125, c2 <= 2^14, eta_m <= 4: certified fast path allowed
+  int32_t cert_ok;   // 2^-28 <= eps <= 2^60, tau >= 2^-125, c2 <= 2^14, eta_m <= 4, kwd <= 1: certified fast path allowed
 };
 
 // The scalars of the certified path's packed operations, twice each: the two
 // halves of an f32x2 operand.
 struct StepPairs {
-  uint64_t b1, b2, omb1, omb2, ka, c2, km, ln2, eps;
+  uint64_t b1, b2, omb1, omb2, ka, c2, km, ln2, eps, kwd;
   uint64_t nc1, nc2, nc0;  // minus the error bound's coefficients
   uint64_t m1;             // -1
 };

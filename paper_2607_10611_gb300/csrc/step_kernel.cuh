@@ -332,6 +332,16 @@ __device__ __forceinline__ f32x2 fma2_rn(f32x2 x, f32x2 y, f32x2 z) {
 // wn' not finite shows as a NaN in `fin` (the product with 0), and the group
 // is then recomputed.
 //
+// Options.  The clamps of n (g_max) and of the weight (w_max) are 1-Lipschitz
+// as well; `fin` sees wn' before w_max.  With decay, u_a becomes fl(u_a -
+// fl(kwd w)), kwd <= 1 (cert_ok), both sides rounding once more: at most
+// 2u (|u_a| + |w|), and |wn'| grows by as much, so rho's coefficient becomes
+// 2.5 2^-22 (|u_a|'s has the room).
+// Before, a list with any option ran the exact sequence throughout: with
+// decay and both clamps 464 M parameters in BF16 took 2188 us, now 1248 (with
+// no option 1235); 217 M: E4M3, SR, binary32 moments 1663 -> 1100 us,
+// block-scaled 1660 -> 1211, NVFP4 2440 -> 1294.
+//
 // The caller stores the encoding of wn' only when encoding wn' - eps (rounded
 // down) and wn' + eps (rounded up) gives the same code: every encoder here is
 // monotone, so the canonical wn, which lies in between, has that code too.
@@ -357,6 +367,7 @@ struct CertPair {
 
 // m, v, ve go in as the stored moments and come back updated; `fin` collects
 // wn' 0 (NaN once any wn' is not finite).
+template <bool OPT>
 __device__ __forceinline__ CertPair madam_cert_pair(const StepScalars& s, const StepPairs& q, float w0, float w1,
                                                     float g0, float g1, float& m0, float& m1, float& v0, float& v1,
                                                     float& e0, float& e1, f32x2& fin) {
@@ -373,12 +384,22 @@ __device__ __forceinline__ CertPair madam_cert_pair(const StepScalars& s, const 
   unpk(fma2_rn(pk(sqrt_approx_ftz(v0), sqrt_approx_ftz(v1)), q.c2, q.eps), d0, d1);
   const f32x2 ua = mul2_rn(mul2_rn(q.ka, m), pk(rcp_approx_ftz(d0), rcp_approx_ftz(d1)));
   unpk(fma2_rn(pk(sqrt_approx_ftz(e0), sqrt_approx_ftz(e1)), q.c2, q.eps), d0, d1);
-  const f32x2 n = mul2_rn(ge, pk(rcp_approx_ftz(d0), rcp_approx_ftz(d1)));
+  f32x2 n = mul2_rn(ge, pk(rcp_approx_ftz(d0), rcp_approx_ftz(d1)));
+  if (OPT && s.gmax_on) {
+    unpk(n, x0, x1);
+    n = pk(fmaxf(-s.gmax, fminf(x0, s.gmax)), fmaxf(-s.gmax, fminf(x1, s.gmax)));
+  }
   const float r0 = fmaxf(fabsf(w0), s.tau), r1 = fmaxf(fabsf(w1), s.tau);
   unpk(mul2_rn(mul2_rn(q.km, n), pk(rcp_approx_ftz(r0), rcp_approx_ftz(r1))), x0, x1);
   const f32x2 um = pk(fmaxf(s.lo, fminf(x0, s.hi)), fmaxf(s.lo, fminf(x1, s.hi)));
-  o.wn = add2_rn(fma2_rn(w, um, w), ua);
+  f32x2 uad = ua;
+  if (OPT && s.wd_on) uad = fma2_rn(mul2_rn(q.kwd, w), q.m1, ua);  // u_a - kwd w (the product with -1 is exact)
+  o.wn = add2_rn(fma2_rn(w, um, w), uad);
   fin = fma2_rn(o.wn, 0ull, fin);
+  if (OPT && s.wmax_on) {
+    unpk(o.wn, x0, x1);
+    o.wn = pk(fmaxf(-s.wmax, fminf(x0, s.wmax)), fmaxf(-s.wmax, fminf(x1, s.wmax)));
+  }
   float a0, a1;
   unpk(mul2_rn(w, um), x0, x1);
   unpk(ua, a0, a1);
@@ -403,14 +424,19 @@ __device__ __forceinline__ bool cert_not_finite(f32x2 fin) {
 
 // The weight of the canonical sequence from the already updated (exact)
 // moments: the exact fallback of the certified path.
+template <bool OPT>
 static __device__ __noinline__ float madam_wn_exact(const StepScalars& s, float w, float g, float m1, float v1,
                                              float ve1) {
-  const float ua = __fdiv_rn(__fmul_rn(s.ka, m1), __fmaf_rn(__fsqrt_rn(v1), s.c2, s.eps));
+  float ua = __fdiv_rn(__fmul_rn(s.ka, m1), __fmaf_rn(__fsqrt_rn(v1), s.c2, s.eps));
+  if (OPT && s.wd_on) ua = __fsub_rn(ua, __fmul_rn(s.kwd, w));
   const float ge = __fmul_rn(__fmul_rn(s.ln2, w), g);
-  const float n = __fdiv_rn(ge, __fmaf_rn(__fsqrt_rn(ve1), s.c2, s.eps));
+  float n = __fdiv_rn(ge, __fmaf_rn(__fsqrt_rn(ve1), s.c2, s.eps));
+  if (OPT && s.gmax_on) n = fmaxf(-s.gmax, fminf(n, s.gmax));
   float um = __fdiv_rn(__fmul_rn(s.km, n), fmaxf(fabsf(w), s.tau));
   um = fmaxf(s.lo, fminf(um, s.hi));
-  return __fadd_rn(__fmaf_rn(w, um, w), ua);
+  float wn = __fadd_rn(__fmaf_rn(w, um, w), ua);
+  if (OPT && s.wmax_on) wn = fmaxf(-s.wmax, fminf(wn, s.wmax));
+  return wn;
 }
 
 // ---------------------------------------------------------------------------
@@ -845,7 +871,7 @@ __device__ __forceinline__ void group_random_bits(const StepArgs& a, uint64_t gi
 // The canonical weight of slot j of consumer c (a runtime index), from the
 // original inputs in the stage at st, which must still be allocated.  dec:
 // the scale its code decodes with (E4M3 formats and NVFP4).
-template <int WD, int GD, int MD>
+template <int WD, int GD, int MD, bool OPT>
 __device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, uint32_t st, int c, int j, float dec) {
   constexpr int GS = esize_of(GD), MS = esize_of(MD);
   const uint32_t i = static_cast<uint32_t>(kGroup * c + j);
@@ -856,7 +882,7 @@ __device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, uint32_t
   auto ld = [&](uint32_t base, int es) -> float {
     return es == 4 ? __uint_as_float(lds_u32(base + 4u * i)) : __uint_as_float(lds_u16(base + 2u * i) << 16);
   };
-  return madam_update<false>(a.s, w, ld(st + a.off_g, GS), ld(st + a.off_m, MS), ld(st + a.off_v, MS),
+  return madam_update<OPT>(a.s, w, ld(st + a.off_g, GS), ld(st + a.off_m, MS), ld(st + a.off_v, MS),
                              ld(st + a.off_ve, MS)).wn;
 }
 
@@ -899,12 +925,12 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
   uint32_t rnd[8];
   if (SR) group_random_bits<WD>(a, static_cast<uint64_t>(x.d.goff + e0), rnd);
 
-  if (WD == kBF16 && !OPT && a.s.cert_ok) {  // certified fast path (see madam_cert_pair)
+  if (WD == kBF16 && a.s.cert_ok) {  // certified fast path (see madam_cert_pair)
     uint32_t ow[4], df[4];  // codes of the lower ends, and where the upper ends' differ (two 16-bit halves each)
     f32x2 fin = 0ull;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+      const CertPair u = madam_cert_pair<OPT>(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
                                          m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
       float l0, l1, h0, h1;
       unpk(add2_rd(u.wn, u.ne), l0, l1);
@@ -927,7 +953,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
 #pragma unroll 1
         for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
           const int j = __ffs(rm) - 1;
-          const float xe = exact_wn_from_stage<WD, GD, MD>(a, st, c, j, 1.0f);
+          const float xe = exact_wn_from_stage<WD, GD, MD, OPT>(a, st, c, j, 1.0f);
           const uint32_t code =
               SR ? (bf16_sr_sum(xe, bf16_element_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j)) >> 16)
                  : (bf16x2_rn(xe, xe) & 0xFFFFu);
@@ -940,7 +966,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
 #pragma unroll
         for (int j = 0; j < kGroup; ++j) {
           if ((redo >> j) & 1u) {
-            const float xe = madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
+            const float xe = madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]);
             const uint32_t code = SR ? (bf16_sr_sum(xe, rnd[j]) >> 16) : (bf16x2_rn(xe, xe) & 0xFFFFu);
             const int sh = 16 * (j & 1);
             ow[j >> 1] = (ow[j >> 1] & ~(0xFFFFu << sh)) | (code << sh);
@@ -949,7 +975,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
       }
     }
     put_bf16(ow, x.d.w, e0, valid, x.vec);
-  } else if (WD == kE4M3 && !OPT && a.s.cert_ok) {
+  } else if (WD == kE4M3 && a.s.cert_ok) {
     // Certified fast path for E4M3: both ends of the bound are scaled by 2^-e
     // with outward rounding and encoded; the largest |w'| must be exact, so an
     // element whose bound may reach the threshold is recomputed as well.  The
@@ -963,7 +989,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
     const f32x2 enc = pk(x.enc_scale, x.enc_scale);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+      const CertPair u = madam_cert_pair<OPT>(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
                                          m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
       const f32x2 l = add2_rd(u.wn, u.ne), h = sub2_ru(u.wn, u.ne, a.p);
       float l0, l1, h0, h1;
@@ -1000,7 +1026,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
           const int j = __ffs(rm) - 1;
           const uint32_t r = SR ? lane32_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j) : 0u;
-          const uint32_t code = exact_code(j, exact_wn_from_stage<WD, GD, MD>(a, st, c, j, x.dec_scale), r);
+          const uint32_t code = exact_code(j, exact_wn_from_stage<WD, GD, MD, OPT>(a, st, c, j, x.dec_scale), r);
           const int sh = 8 * (j & 3);
 #pragma unroll
           for (int i = 0; i < 2; ++i)
@@ -1011,7 +1037,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         for (int j = 0; j < kGroup; ++j) {
           if ((redo >> j) & 1u) {
             const uint32_t code =
-                exact_code(j, madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]), SR ? rnd[j] : 0u);
+                exact_code(j, madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]), SR ? rnd[j] : 0u);
             const int sh = 8 * (j & 3);
             ow[j >> 2] = (ow[j >> 2] & ~(0xFFu << sh)) | (code << sh);
           }
@@ -1124,7 +1150,7 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
   const uint32_t vmask = valid >= kGroup ? 0xFFu : (valid > 0 ? (1u << valid) - 1u : 0u);
   uint32_t ow[2];
   int32_t k_new;
-  if (!OPT && a.s.cert_ok) {
+  if (a.s.cert_ok) {
     // Certified path (see madam_cert_pair).  Keep the fast weights and the
     // thread's largest error bound et; the block maximum then lies in
     // [max |w'| - et, max |w'| + et] (outward rounded).  When both ends give
@@ -1136,7 +1162,7 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
     float nt = 0.0f, am = 0.0f;  // nt = -et
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+      const CertPair u = madam_cert_pair<OPT>(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
                                          m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
       float x0, x1, n0, n1;
       unpk(u.wn, x0, x1);
@@ -1159,8 +1185,8 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
     const bool certain = qlo != 0u && qhi < 0x7E800000u /* 2^126 */ && kl == block_exponent(qhi, k_old);
     k_new = kl;
     auto exact_wn = [&](int j) -> float {
-      if constexpr (STAGED) return exact_wn_from_stage<kE4M3B, GD, MD>(a, st, c, j, fp16_value(h_old));
-      else return madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
+      if constexpr (STAGED) return exact_wn_from_stage<kE4M3B, GD, MD, OPT>(a, st, c, j, fp16_value(h_old));
+      else return madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]);
     };
     if (__any_sync(0xFFFFFFFFu, !certain)) {  // exact block maximum for the undecided quads
       uint32_t amx = 0u;
@@ -1456,7 +1482,7 @@ __device__ __forceinline__ uint32_t pair_max(uint32_t x) {
 // are stored rounded).  L2-only loads: the moments were written by this
 // thread.  Out of line: the call is rare and its pointers would otherwise stay
 // live through the encode.
-template <int GD>
+template <int GD, bool OPT>
 __device__ __noinline__ float fp4_exact_from_global(const StepArgs& a, const TensorCtx& x, int64_t e,
                                                     float d_old) {
   const uint8_t* pw = static_cast<const uint8_t*>(x.d.w) + (e >> 1);
@@ -1472,7 +1498,7 @@ __device__ __noinline__ float fp4_exact_from_global(const StepArgs& a, const Ten
   asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(bm) : "l"(static_cast<const float*>(x.d.m) + e) : "memory");
   asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(bv) : "l"(static_cast<const float*>(x.d.v) + e) : "memory");
   asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(be) : "l"(static_cast<const float*>(x.d.ve) + e) : "memory");
-  return madam_wn_exact(a.s, w, __uint_as_float(bg), __uint_as_float(bm), __uint_as_float(bv), __uint_as_float(be));
+  return madam_wn_exact<OPT>(a.s, w, __uint_as_float(bg), __uint_as_float(bm), __uint_as_float(bv), __uint_as_float(be));
 }
 
 // Where the rare exact branch of finish_fp4 finds an element's inputs:
@@ -1496,11 +1522,11 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
   float d;
   static_assert(SRC != kExactGlobal || MD == kF32, "exact recompute from global needs binary32 moments");
   auto exact_wn = [&](int j) -> float {
-    if constexpr (SRC == kExactStage) return exact_wn_from_stage<kNVFP4, GD, MD>(a, st, c, j, d_old);
-    else if constexpr (SRC == kExactGlobal) return fp4_exact_from_global<GD>(a, x, e0 + j, d_old);
-    else return madam_wn_exact(a.s, w[j], g[j], m[j], v[j], ve[j]);
+    if constexpr (SRC == kExactStage) return exact_wn_from_stage<kNVFP4, GD, MD, OPT>(a, st, c, j, d_old);
+    else if constexpr (SRC == kExactGlobal) return fp4_exact_from_global<GD, OPT>(a, x, e0 + j, d_old);
+    else return madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]);
   };
-  if (!OPT && a.s.cert_ok) {
+  if (a.s.cert_ok) {
     // Certified path, as for block-scaled E4M3: fast weights and one error
     // bound et; the pair's maximum bounds decide the scale code (exact
     // maximum where they do not); then each element's interval, divided by
@@ -1510,7 +1536,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
     f32x2 fin = 0ull;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const CertPair u = madam_cert_pair(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
+      const CertPair u = madam_cert_pair<OPT>(a.s, a.p, w[2 * i], w[2 * i + 1], g[2 * i], g[2 * i + 1], m[2 * i],
                                          m[2 * i + 1], v[2 * i], v[2 * i + 1], ve[2 * i], ve[2 * i + 1], fin);
       float n0, n1;
       unpk(u.wn, wf[2 * i], wf[2 * i + 1]);

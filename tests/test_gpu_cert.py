@@ -91,3 +91,24 @@ def test_block_codes_at_the_ends_of_the_range(md, rnd):
         sc = torch.where((torch.arange(mt.bscale[k].numel()) % 2) == 0, torch.tensor(2.0 ** -10), torch.tensor(2.0 ** 15))
         mt.bscale[k].copy_(sc.to(torch.float16))
     _steps(P().Run(wl, mt=mt, hp=dict(lr_mul=0.5, lr_add=1e-3)), 3, f"ends {md}/{rnd}")
+
+
+# The options' certified path in every weight format: clamps that bind for
+# many elements (so that intervals straddle them), decay up to and past the
+# largest the certificate takes (eta_a lambda = 1), and non-finite inputs,
+# which a clamp would hide
+OPTIONS = [dict(g_max=0.7, w_max=0.02, wd_add=0.1), dict(g_max=1e-3), dict(w_max=1e-3), dict(lr_add=0.5, wd_add=2.0),
+           dict(lr_add=0.5, wd_add=2.5), dict(lr_mul=4.0, lr_add=0.3, wd_add=0.3, g_max=2.0, w_max=0.5)]
+
+
+@pytest.mark.parametrize("hp", OPTIONS)
+@pytest.mark.parametrize("rnd", ["nearest", "stochastic"])
+@pytest.mark.parametrize("name", ["llama_7b", "llama_1p5b", "llama_1p5b_mixed", "llama_1p5b_nvfp4"])
+def test_options_in_every_format(name, rnd, hp):
+    mt = W.materialize(W.replace(W.SMALL[name], moment_dtype="bf16", rounding=rnd), "cpu", warm_state=True)
+    big = max(range(len(mt.g)), key=lambda k: mt.g[k].numel())
+    for i, x in enumerate((float("nan"), float("inf"), -float("inf"))):
+        mt.g[big][100 * i::977] = x
+    mt.ve[big][17::1009] = float("inf")
+    wl = mt.workload
+    _steps(P().Run(wl, mt=mt, hp=hp), 2, f"{name}/{rnd}/{hp}")
