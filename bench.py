@@ -483,8 +483,8 @@ def host_link_ms(h_src, d_dst, h_dst, d_src, stream, reps: int = 3) -> float:
 def run_toy(steps: int):
     """The BF16-stored matrix-fitting diagnostic: every regime with every
     update rule for `steps` steps at n = 4096, B = 65536, through
-    mpadam_toy_run (graph replays).  Reports the mean device time per step
-    (three kernels) and, per run, the mean loss of the last 64 steps over
+    mpadam_toy_run.  Reports the mean device time per step
+    (a run is one cooperative kernel) and, per run, the mean loss of the last 64 steps over
     that of the first 4 (lower is better)."""
     import torch
     import workloads as W
@@ -501,12 +501,12 @@ def run_toy(steps: int):
                               lr_add=lr if mode != "multiplicative" else 0.0,
                               lr_mul=lr if mode != "additive" else 0.0)
             losses = torch.zeros(steps, dtype=torch.float64, device="cuda")
-            d.run(1, 64, losses[:64])           # capture the run graph (not timed)
+            d.run(1, 64, losses[:64])           # warm-up (not timed)
             torch.cuda.synchronize()
             w.copy_(p.w0)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record(stream)
-            d.run(1, steps, losses)             # CUDA-graph replays of 64 steps
+            d.run(1, steps, losses)             # one kernel
             e1.record(stream)
             torch.cuda.synchronize()
             total_ms += e0.elapsed_time(e1)

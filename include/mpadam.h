@@ -427,19 +427,23 @@ int32_t mpadam_toy_create(int64_t n, const mpadam_toy_config* cfg, mpadam_toy_st
 /* One step t (>= 1) on w (device, n BF16 bit patterns, updated in place)
  * towards wstar (device, n binary32 targets), asynchronously on `stream`.
  * loss_out: device double receiving the minibatch loss of this step (before
- * the update), or NULL.  Three kernel launches.  Errors: EINVAL, ECUDA. */
+ * the update), or NULL.  Two kernel launches.  Errors: EINVAL, ECUDA. */
 int32_t mpadam_toy_step(mpadam_toy_state* s, uint16_t* w, const float* wstar, int64_t step, double* loss_out,
                         struct CUstream_st* stream);
 
 /* `steps` consecutive steps first_step, first_step + 1, ... on `stream`, as
  * many mpadam_toy_step calls would give, with the loss of step first_step + i
- * written to losses[i] (device, double[steps]; or NULL).  The step number
- * lives in device memory, advanced by the last kernel of each step, so the
- * steps run as replays of a CUDA graph of 64 steps, captured on an internal
- * stream at the first call with these w, wstar and losses pointers (the
- * remainder runs as plain launches).  Errors: EINVAL, ECUDA. */
+ * written to losses[i] (device, double[steps]; or NULL).  The steps run inside
+ * one cooperative kernel (one per 8192 steps) whose CTAs wait on one another
+ * with bounded waits; mpadam_toy_status says whether one gave up.  Errors:
+ * EINVAL, ECUDA. */
 int32_t mpadam_toy_run(mpadam_toy_state* s, uint16_t* w, const float* wstar, int64_t first_step, int64_t steps,
                        double* losses, struct CUstream_st* stream);
+
+/* Synchronises the device, then reads and clears the state's device error
+ * word: 0, or 1 when a wait inside a run gave up (its results are then not
+ * valid, nor is the state).  Errors: EINVAL, ECUDA. */
+int32_t mpadam_toy_status(mpadam_toy_state* s, int32_t* code);
 
 /* Frees the scratch (synchronises the device first).  NULL is a no-op. */
 int32_t mpadam_toy_destroy(mpadam_toy_state* s);

@@ -23,8 +23,8 @@ ROUNDING = {"nearest": MPADAM_ROUND_NEAREST, "stochastic": MPADAM_ROUND_STOCHAST
 EXPORTED = ["mpadam_create", "mpadam_create_ex", "mpadam_fp8_init", "mpadam_step", "mpadam_step_host",
             "mpadam_destroy", "mpadam_last_error", "mpadam_global_offset", "mpadam_global_length", "mpadam_set_grid",
             "mpadam_set_tail_pool", "mpadam_launch_info", "mpadam_rng_lanes", "mpadam_step_noalloc", "mpadam_noalloc_status", "mpadam_device_status",
-            "mpadam_toy_create", "mpadam_toy_step", "mpadam_toy_run", "mpadam_toy_destroy", "mpadam_host_buffer_alloc",
-            "mpadam_host_buffer_free", "mpadam_debug_fail_allocation", "mpadam_debug_tile_schedule"]
+            "mpadam_toy_create", "mpadam_toy_step", "mpadam_toy_run", "mpadam_toy_status", "mpadam_toy_destroy",
+            "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation", "mpadam_debug_tile_schedule"]
 
 
 class MPAdamError(RuntimeError):
@@ -119,6 +119,7 @@ def lib() -> ctypes.CDLL:
             "mpadam_toy_create": [i64, P, P],
             "mpadam_toy_step": [P, P, P, i64, P, P],
             "mpadam_toy_run": [P, P, P, i64, i64, P, P],
+            "mpadam_toy_status": [P, P],
             "mpadam_toy_destroy": [P],
             "mpadam_host_buffer_alloc": [i64, P],
             "mpadam_host_buffer_free": [P, i64],
@@ -266,6 +267,13 @@ def mpadam_toy_step(state: int, w: int, wstar: int, step: int, loss_out: int = 0
 def mpadam_toy_run(state: int, w: int, wstar: int, first_step: int, steps: int, losses: int = 0,
                    stream: int = 0) -> None:
     _check(lib().mpadam_toy_run(state, w, wstar, first_step, steps, losses or None, stream or None))
+
+
+def mpadam_toy_status(state: int) -> int:
+    """Synchronises; returns and clears the diagnostic's device error word (0 = none)."""
+    out = ctypes.c_int32()
+    _check(lib().mpadam_toy_status(state, ctypes.byref(out)))
+    return out.value
 
 
 def mpadam_toy_destroy(state: int) -> None:

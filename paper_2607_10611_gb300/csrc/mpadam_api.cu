@@ -1361,17 +1361,7 @@ extern "C" int32_t mpadam_noalloc_status(cudaStream_t stream, int32_t* code) {
 struct mpadam_toy_state {
   mpadam::ToyArgs a{};
   int device = 0;
-  int64_t* t_dev = nullptr;           // run mode step counter {t, first t}
-  cudaStream_t cap = nullptr;         // capture stream of the run graph
-  cudaGraphExec_t exec = nullptr;     // kToyGraphSteps steps for the pointers below
-  const void* g_w = nullptr;
-  const void* g_ws = nullptr;
-  const void* g_loss = nullptr;
 };
-
-namespace {
-constexpr int64_t kToyGraphSteps = 64;  // steps per replay of the run graph
-}
 
 extern "C" int32_t mpadam_toy_create(int64_t n, const mpadam_toy_config* cfg, mpadam_toy_state** out) {
   if (!out) return fail(MPADAM_EINVAL, "out is NULL");
@@ -1398,13 +1388,15 @@ extern "C" int32_t mpadam_toy_create(int64_t n, const mpadam_toy_config* cfg, mp
   const size_t B = (size_t)cfg->batch;
   if (dev_malloc(&a.cnt, sizeof(int32_t) * n) != cudaSuccess || dev_malloc(&a.first, sizeof(int32_t) * n) != cudaSuccess ||
       dev_malloc(&a.idx, sizeof(int32_t) * B) != cudaSuccess || dev_malloc(&a.res, sizeof(float) * B) != cudaSuccess ||
-      dev_malloc(&st->t_dev, sizeof(int64_t) * 2) != cudaSuccess ||
+      dev_malloc(&a.sync, sizeof(mpadam::ToySync)) != cudaSuccess ||
+      dev_malloc(&a.loss_hi, sizeof(double) * mpadam::kToyRunSteps) != cudaSuccess || dev_malloc(&a.err, sizeof(int32_t)) != cudaSuccess ||
       dev_malloc(&a.partial, sizeof(double) * (B / 256 + 2)) != cudaSuccess) {
     mpadam_toy_destroy(st);
     return fail(MPADAM_EALLOC, "allocation of the diagnostic's scratch failed");
   }
   if ((e = cudaMemset(a.cnt, 0, sizeof(int32_t) * n)) != cudaSuccess ||
       (e = cudaMemset(a.first, 0, sizeof(int32_t) * n)) != cudaSuccess ||
+      (e = cudaMemset(a.err, 0, sizeof(int32_t))) != cudaSuccess ||
       (e = cudaDeviceSynchronize()) != cudaSuccess) {
     mpadam_toy_destroy(st);
     return cuda_fail(e, "clearing the diagnostic's scratch");
@@ -1460,48 +1452,27 @@ extern "C" int32_t mpadam_toy_run(mpadam_toy_state* s, uint16_t* w, const float*
   a.w = w;
   a.wstar = wstar;
   a.loss_out = nullptr;
-  a.t_dev = s->t_dev;
-  a.loss_base = losses;
-  // the graph of kToyGraphSteps steps, captured once per set of pointers
-  if (steps >= kToyGraphSteps && (!s->exec || s->g_w != w || s->g_ws != wstar || s->g_loss != losses)) {
-    if (s->exec) { cudaGraphExecDestroy(s->exec); s->exec = nullptr; }
-    if (!s->cap && (e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking)) != cudaSuccess)
-      return cuda_fail(e, "cudaStreamCreate");
-    if ((e = cudaStreamBeginCapture(s->cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
-      return cuda_fail(e, "cudaStreamBeginCapture");
-    cudaError_t le = cudaSuccess;
-    for (int64_t i = 0; i < kToyGraphSteps && le == cudaSuccess; ++i) le = mpadam::launch_toy_step(a, s->cap);
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamEndCapture(s->cap, &graph);
-    if (le != cudaSuccess || e != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      return cuda_fail(le != cudaSuccess ? le : e, "capture of the diagnostic's run graph");
-    }
-    e = cudaGraphInstantiate(&s->exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) { s->exec = nullptr; return cuda_fail(e, "cudaGraphInstantiate"); }
-    s->g_w = w;
-    s->g_ws = wstar;
-    s->g_loss = losses;
-  }
-  if ((e = mpadam::launch_toy_set_step(s->t_dev, first_step, stream)) != cudaSuccess)
-    return cuda_fail(e, "launch of the step-counter kernel");
-  int64_t done = 0;
-  for (; s->exec && done + kToyGraphSteps <= steps; done += kToyGraphSteps)
-    if ((e = cudaGraphLaunch(s->exec, stream)) != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
-  for (; done < steps; ++done)
-    if ((e = mpadam::launch_toy_step(a, stream)) != cudaSuccess) return cuda_fail(e, "launch of the diagnostic's kernels");
+  e = mpadam::launch_toy_run(a, first_step, steps, losses, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "launch of the diagnostic's run");
+  return MPADAM_OK;
+}
+
+extern "C" int32_t mpadam_toy_status(mpadam_toy_state* s, int32_t* code) {
+  if (!s || !code) return fail(MPADAM_EINVAL, "NULL argument");
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
+  e = cudaMemcpy(code, s->a.err, sizeof(int32_t), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "reading the error word");
+  e = cudaMemset(s->a.err, 0, sizeof(int32_t));
+  if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
   return MPADAM_OK;
 }
 
 extern "C" int32_t mpadam_toy_destroy(mpadam_toy_state* s) {
   if (!s) return MPADAM_OK;
   cudaDeviceSynchronize();
-  if (s->exec) cudaGraphExecDestroy(s->exec);
-  if (s->cap) cudaStreamDestroy(s->cap);
-  if (s->t_dev) cudaFree(s->t_dev);
   mpadam::ToyArgs& a = s->a;
-  for (void* p : {(void*)a.cnt, (void*)a.first, (void*)a.idx, (void*)a.res, (void*)a.partial})
+  for (void* p : {(void*)a.cnt, (void*)a.first, (void*)a.idx, (void*)a.res, (void*)a.partial, (void*)a.sync, (void*)a.loss_hi, (void*)a.err})
     if (p) cudaFree(p);
   delete s;
   return MPADAM_OK;

@@ -42,11 +42,15 @@ class ToyDiagnostic:
 
     def run(self, first_step: int, steps: int, losses: Optional[torch.Tensor] = None,
             stream: Optional[torch.cuda.Stream] = None):
-        """Steps first_step .. first_step + steps - 1 (CUDA-graph replays);
+        """Steps first_step .. first_step + steps - 1 inside one kernel;
         losses: a CUDA float64 tensor of `steps` elements, or None."""
         s = (stream or torch.cuda.current_stream(self.w.device)).cuda_stream
         N.mpadam_toy_run(self.state, self.w.data_ptr(), self.wstar.data_ptr(), first_step, steps,
                          losses.data_ptr() if losses is not None else 0, s)
+
+    def device_status(self) -> int:
+        """Device error word of the runs so far (0 = none); synchronises."""
+        return N.mpadam_toy_status(self.state)
 
     def close(self):
         if getattr(self, "state", None):
