@@ -140,7 +140,7 @@ struct StepArgs {
   int32_t static_q;          // static prefix of each CTA's range, in 1/1024 (1024 when pool is nullptr)
   int32_t* err;              // DeviceError bits, or nullptr
   const PoolChunk* pool;     // [pool_chunks] tail pool, or nullptr (static ranges only)
-  uint32_t* pool_next;       // next unclaimed pool chunk; zero when the launch starts
+  uint32_t* pool_next;       // next unclaimed pool chunk; zero when the launch starts and again when it ends
   int32_t pool_chunks;
   // Launches of at most kInlineTensors tensors (a flat parameter buffer, a
   // short list) carry their descriptors, aux entries and gradient pointers

@@ -1751,6 +1751,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
   __shared__ int64_t stage_tile[kMaxStages];  // tile the producer put in each stage (-1: no more work)
   __shared__ int32_t stage_k[kMaxStages];     // and its tensor
 
+  // Programmatic dependent launch: the next launch of the stream may start its
+  // own entry (it waits below, like this one, for everything before it).
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int S = a.stages;
@@ -1820,6 +1823,12 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     }
     mbar_init_fence();
     pol = evict_first_policy();
+  }
+  // Nothing of global memory is touched before the work ahead in the stream is
+  // complete: the previous step, the kernels that wrote the gradients or the
+  // tables.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == kConsumers) {
     if (t < t_end) {
       load(first_tensor(a, tb));
       while (t >= d.tile_off + tiles) load(pk + 1);
@@ -1830,11 +1839,15 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
 
   if (warp == kConsumerWarps) {
     if (lane != 0) return;
+    // Every CTA's claims end with one beyond the pool, pool_chunks + gridDim.x
+    // in all: the last of them wraps the counter back to 0 for the next launch
+    // (a memset before every launch cost a gap of its own on the stream).
+    auto claim = [&]() { return atomicInc(a.pool_next, static_cast<uint32_t>(a.pool_chunks) + gridDim.x - 1u); };
     bool failed = false;
     for (;;) {
       if (t >= t_end) {  // static part done: next chunk of the tail pool, if any
         if (!a.pool) break;
-        const uint32_t j = atomicAdd(a.pool_next, 1u);
+        const uint32_t j = claim();
         if (j >= static_cast<uint32_t>(a.pool_chunks)) break;
         const PoolChunk pc = a.pool[j];
         t = pc.start;
@@ -1856,6 +1869,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         if (!mbar_wait(smem_addr(&full_bar[it % S]), static_cast<uint32_t>((it / S) & 1)) && a.err)
           atomicOr(a.err, kErrDrainWait);
       }
+      if (a.pool)
+        while (claim() < static_cast<uint32_t>(a.pool_chunks)) {}  // leave the counter as a CTA that finished would
       return;
     }
     // no more work: once the next stage is free, post the end marker there
