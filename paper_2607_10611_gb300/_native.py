@@ -7,9 +7,11 @@ been built (paper_2607_10611_gb300.build()); there is no fallback.
 """
 from __future__ import annotations
 
+import array
 import ctypes
+import itertools
 import math
-from typing import Optional, Sequence
+from typing import Iterable, Optional, Sequence
 
 from . import builder as _build
 
@@ -145,11 +147,30 @@ def _check(status: int) -> None:
         raise MPAdamError(status, mpadam_last_error())
 
 
-def _ptr_array(ptrs: Sequence[int]):
-    arr = (ctypes.c_void_p * max(1, len(ptrs)))()
-    for i, p in enumerate(ptrs):
-        arr[i] = p
-    return arr
+def _ptr_array(ptrs: Iterable[int]) -> array.array:
+    """Pointers (ints; None = NULL) as 64-bit words; pass buffer_info()[0] while the array lives."""
+    ptrs = list(ptrs)
+    try:
+        return array.array("Q", ptrs)
+    except (TypeError, OverflowError):  # None, ctypes pointers, negative ints: as ctypes converts them
+        arr = (ctypes.c_void_p * max(1, len(ptrs)))()
+        for i, p in enumerate(ptrs):
+            arr[i] = p
+        return array.array("Q", bytes(arr)[:8 * len(ptrs)])
+
+
+def _tensor_table(tensors: Sequence[tuple]) -> array.array:
+    """(w, m, v, ve, numel) per tensor as an array of mpadam_tensor (five 64-bit words each)."""
+    try:
+        arr = array.array("Q", itertools.chain.from_iterable(tensors))
+        if len(arr) == 5 * len(tensors) and all(len(t) == 5 for t in tensors):
+            return arr
+    except (TypeError, OverflowError):  # None, a negative size: as ctypes converts them
+        pass
+    arr = (mpadam_tensor * max(1, len(tensors)))()
+    for i, (w, m, v, ve, n) in enumerate(tensors):
+        arr[i] = mpadam_tensor(w, m, v, ve, n)
+    return array.array("Q", bytes(arr)[:ctypes.sizeof(mpadam_tensor) * len(tensors)])
 
 
 def mpadam_create(tensors: Sequence[tuple], cfg: mpadam_config, fp8_exp: int = 0, fp8_amax: int = 0) -> int:
@@ -185,13 +206,15 @@ def mpadam_fp8_init(state: int, init_exp: Sequence[int], first_step: int, stream
 
 
 def mpadam_step(state: int, grads: Sequence[int], step: int, stream: int = 0) -> None:
-    _check(lib().mpadam_step(state, _ptr_array(grads), step, stream or None))
+    """grads: one pointer per tensor; an array.array("Q") of them is passed as it is."""
+    arr = grads if type(grads) is array.array and grads.typecode == "Q" else _ptr_array(grads)
+    _check(lib().mpadam_step(state, arr.buffer_info()[0], step, stream or None))
 
 
 def mpadam_step_host(state: int, host_grads: Sequence[int], host_w_out: Sequence[int], step: int,
                      stream: int = 0) -> None:
-    _check(lib().mpadam_step_host(state, _ptr_array(host_grads), _ptr_array(host_w_out), step,
-                                  stream or None))
+    g, w = _ptr_array(host_grads), _ptr_array(host_w_out)
+    _check(lib().mpadam_step_host(state, g.buffer_info()[0], w.buffer_info()[0], step, stream or None))
 
 
 def mpadam_destroy(state: int) -> None:
@@ -239,10 +262,8 @@ def mpadam_rng_lanes(seed: int, step: int, weight_dtype: int, first: int, n: int
 def mpadam_step_noalloc(tensors: Sequence[tuple], grads: Sequence[int], cfg: mpadam_config, step: int,
                         fp8_exp: int = 0, fp8_amax: int = 0, stream: int = 0) -> None:
     """Allocation-free step: tensors as for mpadam_create, grads as for mpadam_step."""
-    arr = (mpadam_tensor * max(1, len(tensors)))()
-    for i, (w, m, v, ve, n) in enumerate(tensors):
-        arr[i] = mpadam_tensor(w, m, v, ve, n)
-    _check(lib().mpadam_step_noalloc(arr, len(tensors), _ptr_array(grads), ctypes.byref(cfg),
+    arr, g = _tensor_table(tensors), _ptr_array(grads)
+    _check(lib().mpadam_step_noalloc(arr.buffer_info()[0], len(tensors), g.buffer_info()[0], ctypes.byref(cfg),
                                      fp8_exp or None, fp8_amax or None, step, stream or None))
 
 

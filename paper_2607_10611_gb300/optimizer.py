@@ -11,6 +11,7 @@ element count of every tensor is taken from its first moment.
 """
 from __future__ import annotations
 
+import array
 from typing import List, Optional, Sequence
 
 import torch
@@ -20,6 +21,19 @@ from . import _native as N
 _STORAGE = {"bf16": torch.bfloat16, "e4m3": torch.uint8, "e4m3_b32": torch.uint8, "nvfp4": torch.uint8,
             "f32": torch.float32}
 _SCALES = {"e4m3_b32": torch.float16, "nvfp4": torch.uint8}
+
+
+def _pointers(tensors) -> array.array:
+    """Device pointers of tensors, as the array that the C ABI takes."""
+    try:
+        return array.array("Q", map(torch.Tensor.data_ptr, tensors))
+    except TypeError:  # not torch tensors: anything with a data_ptr()
+        return array.array("Q", [t.data_ptr() for t in tensors])
+
+
+def _raw_stream(device: torch.device) -> int:
+    """Handle of the device's current stream (without the Stream object, which costs 2 us)."""
+    return torch._C._cuda_getCurrentRawStream(device.index)
 
 
 class HostBuffer:
@@ -107,8 +121,10 @@ class MPAdam:
 
     # -- steps ---------------------------------------------------------------
     def step(self, grads: Sequence[torch.Tensor], t: int, stream: Optional[torch.cuda.Stream] = None):
-        s = (stream or torch.cuda.current_stream(self.device)).cuda_stream
-        N.mpadam_step(self.state, [g.data_ptr() for g in grads], t, s)
+        # The host's share of a short list's step: pointers go straight into one array of words, and the current
+        # stream comes as its raw handle (98 tensors: 19.0 us per call before, see _raw_stream and _pointers).
+        s = stream.cuda_stream if stream else _raw_stream(self.device)
+        N.mpadam_step(self.state, _pointers(grads), t, s)
 
     def step_ptrs(self, grad_ptrs: Sequence[int], t: int, stream: int):
         N.mpadam_step(self.state, grad_ptrs, t, stream)
