@@ -1002,17 +1002,31 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
     }
     uint32_t redo = e4m3_interval_codes<SR>(lo, hi, rnd, ow);
     const float sat = __fmul_rn(448.0f, x.cc_scale);  // 448 2^e: from here on codes saturate
-    if (top >= fminf(amax_f, sat) || cert_not_finite(fin)) {
-      if (!(top < sat) || cert_not_finite(fin)) {
+    const bool past = !(top < sat) || cert_not_finite(fin);
+    const bool cand = past || top >= amax_f;
+    if (STAGED ? __any_sync(0xFFFFFFFFu, cand) : cand) {
+      // Maximum candidates by code: |w'| lies above the value of code - 1 and
+      // below that of code + 1.  So |w'| >= amax_f has a code at or above
+      // amax_f's own, rounded down, and (whole warps) the warp's largest has a
+      // code at or above the warp's largest code - 1.  A warp's first group of
+      // a tensor, whose threshold is still zero, recomputes a few elements
+      // instead of all 256 (a 1 Mi list 13.4 -> 9.4 us, 5 M 28.5 -> 24.5).
+      uint32_t cm = 0u;
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) {
+        const uint32_t cj = (ow[j >> 2] >> (8 * (j & 3))) & 0x7Fu;
+        if (!past && !((redo >> j) & 1u)) cm = max(cm, cj);
+      }
+      if (STAGED) cm = __reduce_max_sync(0xFFFFFFFFu, cm);
+      if (past) {
         redo = 0xFFu;
-      } else {
-        // maximum candidates: |w'| >= amax_f has a code at or above amax_f's own, rounded down
-        const float A = __fmul_rz(amax_f, x.enc_scale);
-        const uint32_t ab = __float_as_uint(A);
+      } else if (cand) {
+        const uint32_t ab = __float_as_uint(__fmul_rz(amax_f, x.enc_scale));
         const uint32_t ca = ab >= 0x3C800000u ? (ab >> 20) - 960u : 0u;
+        const uint32_t least = max(ca, cm > 0u ? cm - 1u : 0u);
 #pragma unroll
         for (int j = 0; j < kGroup; ++j)
-          if (((ow[j >> 2] >> (8 * (j & 3))) & 0x7Fu) >= ca) redo |= 1u << j;
+          if (((ow[j >> 2] >> (8 * (j & 3))) & 0x7Fu) >= least) redo |= 1u << j;
       }
     }
     if (redo) {  // rare: the canonical weight of undecided elements and maximum candidates
