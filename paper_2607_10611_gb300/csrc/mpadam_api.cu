@@ -207,8 +207,9 @@ int32_t make_geometry(const mpadam_config& c, int32_t wd, int dev, Geometry* g) 
   const int32_t rs = wd == MPADAM_E4M3_B32 ? mpadam::kTileBlocks * 2           // 240 bytes, a 16-byte multiple
                    : wd == MPADAM_NVFP4    ? mpadam::kTileFp4Blocks               // 240 bytes
                                            : 0;
-  g->off_g = rw;
-  g->off_m = rw + rg;
+  // one-byte weights and gradients keep their place modulo 16 bytes: up to a line more
+  g->off_g = rw + (wd == MPADAM_E4M3 || wd == MPADAM_E4M3_B32 ? 16 : 0);
+  g->off_m = g->off_g + rg + 16;
   g->off_v = g->off_m + rm;
   g->off_ve = g->off_v + rm;
   g->off_s = g->off_ve + rm;
@@ -314,6 +315,8 @@ struct Group {
   std::vector<int64_t> numel;     // of its tensors, in order
   bool aux = false;               // the launch reads the aux table
   const void* kernel = nullptr;
+  const void* kernel_mis = nullptr;     // the instance for misaligned gradients or one-byte weights
+  bool w_mis = false;                   // one-byte weights among them that are not 16-byte aligned
   Geometry geo;
   int32_t default_grid = 0, grid = 0;
   int32_t* d_cta_first = nullptr;
@@ -534,11 +537,11 @@ StepArgs base_args(const mpadam_state* s, const Group& g) {
   return a;
 }
 
-const void* select_kernel(const mpadam_config& c, int32_t wd) {
+const void* select_kernel(const mpadam_config& c, int32_t wd, bool mis) {
   const int opt = kernel_options(c) ? 1 : 0;
-  if (wd == MPADAM_BF16) return mpadam::step_kernel_bf16(c.grad_dtype, c.moment_dtype, c.rounding, opt);
-  if (wd == MPADAM_E4M3) return mpadam::step_kernel_e4m3(c.grad_dtype, c.moment_dtype, c.rounding, opt);
-  if (wd == MPADAM_E4M3_B32) return mpadam::step_kernel_e4m3b(c.grad_dtype, c.moment_dtype, c.rounding, opt);
+  if (wd == MPADAM_BF16) return mpadam::step_kernel_bf16(c.grad_dtype, c.moment_dtype, c.rounding, opt, mis);
+  if (wd == MPADAM_E4M3) return mpadam::step_kernel_e4m3(c.grad_dtype, c.moment_dtype, c.rounding, opt, mis);
+  if (wd == MPADAM_E4M3_B32) return mpadam::step_kernel_e4m3b(c.grad_dtype, c.moment_dtype, c.rounding, opt, mis);
   if (wd == MPADAM_NVFP4) return mpadam::step_kernel_nvfp4(c.grad_dtype, c.moment_dtype, c.rounding, opt);
   return nullptr;
 }
@@ -673,11 +676,15 @@ int32_t create_state(const std::vector<TensorIn>& t, const mpadam_config* cfg, i
     if (e != cudaSuccess) { release(s); return cuda_fail(e, "cudaDeviceGetAttribute"); }
     int32_t rc;
     for (auto& g : s->groups) {
-      g.kernel = select_kernel(*cfg, g.wd);
-      if (!g.kernel) { release(s); return fail(MPADAM_EUNSUPPORTED, "no kernel for these formats"); }
+      g.kernel = select_kernel(*cfg, g.wd, false);
+      g.kernel_mis = select_kernel(*cfg, g.wd, true);
+      for (const TensorDesc& d : g.h_desc)
+        g.w_mis = g.w_mis || ((g.wd == MPADAM_E4M3 || g.wd == MPADAM_E4M3_B32) && d.numel > 0 && !is_aligned(d.w, 16));
+      if (!g.kernel || !g.kernel_mis) { release(s); return fail(MPADAM_EUNSUPPORTED, "no kernel for these formats"); }
       rc = make_geometry(*cfg, g.wd, s->device, &g.geo);
       if (rc) { release(s); return rc; }
-      rc = prepare_kernel(g.kernel, g.geo, s->sm_count, &g.default_grid);
+      rc = prepare_kernel(g.kernel_mis, g.geo, s->sm_count, &g.default_grid);
+      if (!rc) rc = prepare_kernel(g.kernel, g.geo, s->sm_count, &g.default_grid);
       if (rc) { release(s); return rc; }
     }
 
@@ -785,7 +792,10 @@ int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t 
   }
   fill_step(a, s->cfg, step);
   void* params[] = {&a};
-  cudaError_t e = launch_kernel(g.kernel, grid, params, g.geo.dyn_smem, stream);
+  bool mis = g.w_mis;
+  for (int32_t p = g.first; !mis && p < g.first + g.count; ++p)
+    mis = s->numel[s->order[p]] > 0 && !is_aligned(s->h_grads[p], 16);
+  cudaError_t e = launch_kernel(mis ? g.kernel_mis : g.kernel, grid, params, g.geo.dyn_smem, stream);
   if (e != cudaSuccess) return cuda_fail(e, "launch of the step kernel");
   return MPADAM_OK;
 }
@@ -1285,7 +1295,10 @@ extern "C" int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, 
   int sms = 0;
   rc = noalloc_setup(dev, &scratch, &sms);
   if (rc) return rc;
-  const void* kernel = select_kernel(*cfg, cfg->weight_dtype);
+  bool mis = false;
+  for (int32_t k = 0; k < n && !mis; ++k)
+    mis = tensors[k].numel > 0 && (!is_aligned(grads[k], 16) || (wsz == 1 && !is_aligned(tensors[k].w, 16)));
+  const void* kernel = select_kernel(*cfg, cfg->weight_dtype, mis);
   if (!kernel) return fail(MPADAM_EUNSUPPORTED, "no kernel for these formats");
   Geometry geo;
   rc = make_geometry(*cfg, cfg->weight_dtype, dev, &geo);

@@ -153,11 +153,11 @@ struct StepArgs {
 };
 
 // Kernel entry for the given formats (grad f32/bf16, moments f32/bf16,
-// rounding nearest/stochastic, optional clips/decay present); defined in
-// step_bf16.cu / step_e4m3.cu.
-const void* step_kernel_bf16(int grad_dtype, int moment_dtype, int stochastic, int options);
-const void* step_kernel_e4m3(int grad_dtype, int moment_dtype, int stochastic, int options);
-const void* step_kernel_e4m3b(int grad_dtype, int moment_dtype, int stochastic, int options);
+// rounding nearest/stochastic, optional clips/decay present, misaligned
+// gradients or one-byte weights among the tensors); defined in step_*.cu.
+const void* step_kernel_bf16(int grad_dtype, int moment_dtype, int stochastic, int options, bool misaligned);
+const void* step_kernel_e4m3(int grad_dtype, int moment_dtype, int stochastic, int options, bool misaligned);
+const void* step_kernel_e4m3b(int grad_dtype, int moment_dtype, int stochastic, int options, bool misaligned);
 const void* step_kernel_nvfp4(int grad_dtype, int moment_dtype, int stochastic, int options);
 
 }  // namespace mpadam

@@ -3,23 +3,28 @@
 
 namespace mpadam {
 
-template <int GD, int MD, bool SR>
+template <int GD, int MD, bool SR, bool MIS>
 static const void* pick_e4m3(int options) {
-  return options ? reinterpret_cast<const void*>(&step_kernel<kE4M3, GD, MD, SR, true>)
-                 : reinterpret_cast<const void*>(&step_kernel<kE4M3, GD, MD, SR, false>);
+  return options ? reinterpret_cast<const void*>(&step_kernel<kE4M3, GD, MD, SR, true, MIS>)
+                 : reinterpret_cast<const void*>(&step_kernel<kE4M3, GD, MD, SR, false, MIS>);
 }
 
-template <int GD, int MD>
+template <int GD, int MD, bool MIS>
 static const void* pick_e4m3(int sr, int options) {
-  return sr ? pick_e4m3<GD, MD, true>(options) : pick_e4m3<GD, MD, false>(options);
+  return sr ? pick_e4m3<GD, MD, true, MIS>(options) : pick_e4m3<GD, MD, false, MIS>(options);
 }
 
-const void* step_kernel_e4m3(int gd, int md, int sr, int options) {
-  if (gd == kF32 && md == kF32) return pick_e4m3<kF32, kF32>(sr, options);
-  if (gd == kF32 && md == kBF16) return pick_e4m3<kF32, kBF16>(sr, options);
-  if (gd == kBF16 && md == kF32) return pick_e4m3<kBF16, kF32>(sr, options);
-  if (gd == kBF16 && md == kBF16) return pick_e4m3<kBF16, kBF16>(sr, options);
+template <bool MIS>
+static const void* pick_e4m3_formats(int gd, int md, int sr, int options) {
+  if (gd == kF32 && md == kF32) return pick_e4m3<kF32, kF32, MIS>(sr, options);
+  if (gd == kF32 && md == kBF16) return pick_e4m3<kF32, kBF16, MIS>(sr, options);
+  if (gd == kBF16 && md == kF32) return pick_e4m3<kBF16, kF32, MIS>(sr, options);
+  if (gd == kBF16 && md == kBF16) return pick_e4m3<kBF16, kBF16, MIS>(sr, options);
   return nullptr;
+}
+
+const void* step_kernel_e4m3(int gd, int md, int sr, int options, bool mis) {
+  return mis ? pick_e4m3_formats<true>(gd, md, sr, options) : pick_e4m3_formats<false>(gd, md, sr, options);
 }
 
 }  // namespace mpadam

@@ -4,7 +4,7 @@
 // (one per SM) is a producer/consumer pipeline over its tiles:
 //   - one producer warp (one elected lane) picks each tile -- the next of its
 //     own range, then chunks claimed from the launch's tail pool -- posts the
-//     tile and its tensor beside the stage, and streams the tile's slice of
+//     tile and what is needed of its tensor beside the stage, and streams the tile's slice of
 //     every array (weights w, gradients g and the moments mu, nu, nu_e, each
 //     one contiguous run of bytes) into a multi-stage shared-memory ring with
 //     1-D TMA bulk copies (cp.async.bulk ... mbarrier::complete_tx), evict-
@@ -17,10 +17,10 @@
 //     Philox4x32-10 bits) and store w, mu, nu, nu_e straight back to HBM with
 //     vector stores (256-bit for binary32 arrays), then release the stage.
 // Memory latency is hidden by the ring, not by occupancy, so the consumers'
-// instruction stream is the only other limit.  Tensor tails that are not a
-// whole number of 16-byte chunks, and tensors whose pointers are not 16-byte
-// aligned, are read by the consumers directly from global memory with the
-// same arithmetic.  No tensor cores: nothing here is a contraction.
+// instruction stream is the only other limit.  A tensor's last bytes
+// that are not a whole 16-byte line, and tensors with misaligned weights or
+// moments, are read by the consumers directly from global memory with the
+// same arithmetic; misaligned gradients go through the ring all the same.  No tensor cores: nothing here is a contraction.
 //
 // Numerics: every floating-point operation of the canonical sequence is an
 // explicit round-to-nearest intrinsic (__fmul_rn, __fadd_rn, __fmaf_rn,
@@ -45,33 +45,8 @@ namespace mpadam {
 constexpr uint32_t kSpinLimit = 1u << 22;  // mbarrier try_wait attempts before giving up (seconds)
 
 // ---------------------------------------------------------------------------
-// Global memory: streaming vector loads/stores (no L1 allocation).
+// Global memory: streaming vector stores (no L1 allocation).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void ld8(const void* p, uint32_t (&r)[8]) {
-  asm("ld.global.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld8_ro(const void* p, uint32_t (&r)[8]) {
-  asm("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld4(const void* p, uint32_t (&r)[4]) {
-  asm("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld4_ro(const void* p, uint32_t (&r)[4]) {
-  asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-      : "l"(p));
-}
-__device__ __forceinline__ void ld2(const void* p, uint32_t (&r)[2]) {
-  asm("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "l"(p));
-}
 // 256-bit stores carry the binary32 moments (nothing else uses them).  HINT
 // adds an L2 evict-first policy, chosen per kernel instance as measured (two
 // or three alternating runs each): with it the 1.5B list ran 1.4 % faster,
@@ -139,6 +114,15 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
   return v;
 }
+__device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u16(uint32_t addr, uint32_t v) {
+  asm volatile("{\n .reg .b16 h;\n cvt.u16.u32 h, %1;\n st.shared.u16 [%0], h;\n}" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u8(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -148,9 +132,8 @@ __device__ __forceinline__ void mbar_init_fence() {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -653,62 +636,101 @@ __device__ __forceinline__ uint32_t staged_bytes(const void* base, int count, in
   return aligned(base, 16) ? (static_cast<uint32_t>(count * esize) & ~15u) : 0u;
 }
 
+// Gradients may start anywhere and one-byte weights at any multiple of 8 (a
+// reducer's bucket packs gradients without padding; a flat buffer puts tensors
+// at multiples of 8 elements).  A launch with any such array runs the MIS
+// instance of the kernel (read element by element, a list of 4000 ragged
+// tensors in BF16 took 655 us with its gradients in a bucket, now 395; E4M3
+// with BF16 moments in a flat buffer 752, now 374).  It is an instance of its
+// own because its code, though skipped for aligned arrays, slowed short
+// launches by 3 to 7 % and NVFP4 with SR by 4 %; NVFP4 has none and reads them
+// in the element-wise path.  Such an array keeps its place modulo 16 in its
+// region of the stage, `misalign` bytes in (tiles start at multiples of 16
+// bytes from the base, so that is one number per tensor); the copy covers the
+// whole 16-byte lines that lie inside the array, [lo, hi) from the region's
+// start (lo | hi << 16), so only a tensor's first and last group can miss
+// bytes, which patch_group fills in.
+__device__ __forceinline__ uint32_t misalign(const void* base) {
+  return static_cast<uint32_t>(reinterpret_cast<uintptr_t>(base) & 15u);
+}
+__device__ __forceinline__ uint32_t staged_range(const void* base, int64_t numel, int64_t e0, int count, int esize) {
+  const uintptr_t b = reinterpret_cast<uintptr_t>(base);
+  if ((b & 15u) == 0u) return (static_cast<uint32_t>(count * esize) & ~15u) << 16;
+  const uintptr_t a0 = b + static_cast<uintptr_t>(e0) * esize, a1 = a0 + static_cast<uintptr_t>(count) * esize;
+  const uintptr_t line = a0 & ~static_cast<uintptr_t>(15);  // the region's start
+  const uintptr_t first = (b + 15) & ~static_cast<uintptr_t>(15);
+  const uintptr_t last = (b + static_cast<uintptr_t>(numel) * esize) & ~static_cast<uintptr_t>(15);
+  const uintptr_t lo = line > first ? line : first;
+  const uintptr_t up = (a1 + 15) & ~static_cast<uintptr_t>(15);
+  const uintptr_t hi = up < last ? up : last;
+  return hi > lo ? static_cast<uint32_t>(lo - line) | static_cast<uint32_t>(hi - line) << 16 : 0u;
+}
+// Whether bytes [off, off + n) of a region were copied.
+__device__ __forceinline__ bool in_range(uint32_t range, uint32_t off, uint32_t n) {
+  return off >= (range & 0xFFFFu) && off + n <= (range >> 16);
+}
+
 // ---------------------------------------------------------------------------
-// Group loads: 8 consecutive elements from shared memory (staged) or global.
+// Group loads: 8 consecutive elements from the stage.
 // ---------------------------------------------------------------------------
-template <bool RO>
-__device__ __forceinline__ void get_bf16(float (&x)[8], bool staged, uint32_t saddr, const void* g,
-                                         int64_t e0, int valid, bool vec) {
-  if (staged || (vec && valid == kGroup)) {
-    uint32_t r[4];
-    if (staged) lds4(saddr, r);
-    else if (RO) ld4_ro(static_cast<const uint16_t*>(g) + e0, r);
-    else ld4(static_cast<const uint16_t*>(g) + e0, r);
+// The same from an address that is only a multiple of the element size.
+__device__ __forceinline__ void get_bf16_at(float (&x)[8], uint32_t saddr) {
+  uint32_t w[5];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { x[2 * i] = bf16_lo(r[i]); x[2 * i + 1] = bf16_hi(r[i]); }
-  } else {
+  for (int i = 0; i < 5; ++i) w[i] = lds_u32((saddr & ~3u) + 4u * i);
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j)
-      x[j] = j < valid ? __uint_as_float(static_cast<uint32_t>(static_cast<const uint16_t*>(g)[e0 + j]) << 16)
-                       : 0.0f;
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t r = __funnelshift_r(w[i], w[i + 1], (saddr & 2u) * 8u);
+    x[2 * i] = bf16_lo(r);
+    x[2 * i + 1] = bf16_hi(r);
+  }
+}
+__device__ __forceinline__ void get_f32_at(float (&x)[8], uint32_t saddr) {
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) x[j] = __uint_as_float(lds_u32(saddr + 4u * j));
+}
+__device__ __forceinline__ void get_bf16(float (&x)[8], uint32_t saddr) {
+  uint32_t r[4];
+  lds4(saddr, r);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { x[2 * i] = bf16_lo(r[i]); x[2 * i + 1] = bf16_hi(r[i]); }
+}
+__device__ __forceinline__ void get_f32(float (&x)[8], uint32_t saddr) {
+  uint32_t a[4], b[4];
+  lds4(saddr, a);
+  lds4(saddr + 16, b);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { x[i] = __uint_as_float(a[i]); x[4 + i] = __uint_as_float(b[i]); }
+}
+// Eight packed E2M1 codes (element j in bits [4j, 4j + 4)) -> binary32, with
+// the hardware E2M1 -> FP16 conversion (exact) and FP16 -> binary32.
+__device__ __forceinline__ void e2m1x8_to_f32(uint32_t packed, float (&x)[8]) {
+  uint32_t h[4];
+  asm("{\n .reg .b8 b0, b1, b2, b3;\n mov.b32 {b0, b1, b2, b3}, %4;\n"
+      " cvt.rn.f16x2.e2m1x2 %0, b0;\n cvt.rn.f16x2.e2m1x2 %1, b1;\n"
+      " cvt.rn.f16x2.e2m1x2 %2, b2;\n cvt.rn.f16x2.e2m1x2 %3, b3;\n}"
+      : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3])
+      : "r"(packed));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[i]));
+    x[2 * i] = f.x;
+    x[2 * i + 1] = f.y;
   }
 }
 
-template <bool RO>
-__device__ __forceinline__ void get_f32(float (&x)[8], bool staged, uint32_t saddr, const void* g,
-                                        int64_t e0, int valid, bool vec) {
-  if (staged) {
-    uint32_t a[4], b[4];
-    lds4(saddr, a);
-    lds4(saddr + 16, b);
+// Eight NVFP4 weights decoded with d, as one 32-bit word.
+__device__ __forceinline__ void get_fp4(float (&w)[8], uint32_t saddr, float d) {
+  e2m1x8_to_f32(lds_u32(saddr), w);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { x[i] = __uint_as_float(a[i]); x[4 + i] = __uint_as_float(b[i]); }
-  } else if (vec && valid == kGroup) {
-    uint32_t r[8];
-    if (RO) ld8_ro(static_cast<const float*>(g) + e0, r);
-    else ld8(static_cast<const float*>(g) + e0, r);
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) x[j] = __uint_as_float(r[j]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) x[j] = j < valid ? static_cast<const float*>(g)[e0 + j] : 0.0f;
-  }
+  for (int j = 0; j < kGroup; ++j) w[j] = __fmul_rn(w[j], d);
 }
-
-__device__ __forceinline__ void get_e4m3(float (&x)[8], bool staged, uint32_t saddr, const void* g,
-                                         int64_t e0, int valid, bool vec, float scale) {
-  if (staged || (vec && valid == kGroup)) {
-    uint32_t r[2];
-    if (staged) lds2(saddr, r);
-    else ld2(static_cast<const uint8_t*>(g) + e0, r);
-    e4m3x8_to_f32(r, x);
+__device__ __forceinline__ void get_e4m3(float (&x)[8], uint32_t saddr, float scale) {
+  uint32_t r[2];
+  lds2(saddr, r);
+  e4m3x8_to_f32(r, x);
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j) x[j] = __fmul_rn(x[j], scale);
-  } else {
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j)
-      x[j] = j < valid ? __fmul_rn(e4m3_value(static_cast<const uint8_t*>(g)[e0 + j]), scale) : 0.0f;
-  }
+  for (int j = 0; j < kGroup; ++j) x[j] = __fmul_rn(x[j], scale);
 }
 
 // Group stores (vector when whole and aligned, else element by element).
@@ -768,13 +790,37 @@ __device__ __forceinline__ int first_tensor(const StepArgs& a, int64_t tb) {
   return k;
 }
 
+// What the producer posts beside each stage: the tile, and everything the
+// consumers need of its tensor.  The producer's loads of the tables run ahead
+// by the depth of the ring; with the consumers loading them at every change of
+// tensor, each of fifteen warps waited about 1.2 us for two (E4M3: three)
+// dependent reads.
+struct StageHead {
+  void *w, *m, *v, *ve;
+  const void* g;
+  void* scale;       // block scales
+  uint16_t* cc;      // compute copy
+  int64_t goff;
+  int64_t e0;        // the tile's first element
+  int32_t k;         // tensor (-1: no more work)
+  int32_t count;     // elements in the tile
+  int32_t rot;       // the warp that takes the tile's first 256 elements (the following ones follow, cyclically)
+  int32_t ring;
+  float gscale;
+  int32_t e_cur;     // kE4M3: this step's exponent, the maximum that sets the next one, and a lower bound
+  uint32_t amax;     // of this step's maximum so far
+  uint32_t seed;
+  uint32_t w_range, g_range;  // what was copied of the weights (not kNVFP4) and gradients (staged_range)
+};
+static_assert(sizeof(StageHead) * kMaxStages + 16 * kMaxStages <= 1024, "static shared memory (make_geometry leaves 1 KB)");
+
 // Per-tensor values the consumers keep while walking a tensor's tiles.
 struct TensorCtx {
-  TensorDesc d;
-  const void* g;
-  int64_t tiles;
-  bool vec;            // all pointers aligned for vector access by whole groups
-  bool fast;           // every array 16-byte aligned: whole warps of a tile are staged, stored with vector stores
+  TensorDesc d;        // w, m, v, ve, goff, ring
+  const void* g;       // kNVFP4's exact branch (the others read gradients from the stage, or through its head)
+  uint32_t gsh, wsh;   // MIS: misalign() of the gradients and of one-byte weights
+  bool vec;            // every array that is written is aligned for vector stores of whole groups
+  bool fast;           // whole warps of a tile are staged, and stored with vector stores
   float dec_scale, enc_scale;
   float cc_scale;      // E4M3 per-tensor: 2^e of the new encode (compute copy)
   void* scale;         // kE4M3B (FP16) / kNVFP4 (E4M3) block scales
@@ -783,30 +829,129 @@ struct TensorCtx {
   float amax_seed;     // kE4M3: a lower bound of the tensor's largest exact |w'| of this step
 };
 
-template <int WD, int GD, int MD>
-__device__ __forceinline__ void load_tensor(const StepArgs& a, int k, TensorCtx& c) {
-  c.d = desc_of(a, k);
-  c.g = grad_of(a, k);
-  c.tiles = (c.d.numel + kTile - 1) / kTile;
-  c.vec = aligned(c.d.w, WD == kBF16 ? 16 : (WD == kNVFP4 ? 4 : 8)) && aligned(c.g, GD == kF32 ? 32 : 16) &&
-          aligned(c.d.m, MD == kF32 ? 32 : 16) && aligned(c.d.v, MD == kF32 ? 32 : 16) &&
-          aligned(c.d.ve, MD == kF32 ? 32 : 16);
-  c.fast = c.vec && aligned(c.d.w, 16) && aligned(c.g, 16) && aligned(c.d.m, 16) && aligned(c.d.v, 16) &&
-           aligned(c.d.ve, 16);
+template <int WD, int GD, int MD, bool MIS>
+__device__ __forceinline__ void load_tensor(const StageHead& h, TensorCtx& c) {
+  c.d.w = h.w;
+  c.d.m = h.m;
+  c.d.v = h.v;
+  c.d.ve = h.ve;
+  c.d.goff = h.goff;
+  c.d.ring = h.ring;
+  c.g = h.g;
+  c.gsh = MIS ? misalign(h.g) : 0u;
+  c.wsh = MIS && (WD == kE4M3 || WD == kE4M3B) ? misalign(h.w) : 0u;
+  c.vec = aligned(c.d.w, WD == kBF16 ? 16 : (WD == kNVFP4 ? 4 : 8)) && aligned(c.d.m, MD == kF32 ? 32 : 16) &&
+          aligned(c.d.v, MD == kF32 ? 32 : 16) && aligned(c.d.ve, MD == kF32 ? 32 : 16);
+  c.fast = c.vec && (MIS || (aligned(c.d.w, 16) && aligned(c.g, 16)));
   c.dec_scale = c.enc_scale = c.cc_scale = 1.0f;
   c.scale = nullptr;
   c.cc = nullptr;
   c.gscale = 1.0f;
   c.amax_seed = 0.0f;
-  if (WD != kBF16 && a.aux) {  // the launch has aux entries (inline ones too, when it carries its tables)
-    const TensorAux x = aux_of(a, k);
-    c.scale = x.scale;
-    c.cc = x.compute;
-    c.gscale = x.gscale;
+  if (WD != kBF16) {
+    c.scale = h.scale;
+    c.cc = h.cc;
+    c.gscale = h.gscale;
     // the compute copy joins the vector path only when 16-byte aligned;
     // block scales are staged (whole tiles: 240 bytes) only when 16-byte aligned
     if (c.cc && !aligned(c.cc, 16)) c.vec = c.fast = false;
     if ((WD == kE4M3B || WD == kNVFP4) && !aligned(c.scale, 16)) c.fast = false;
+  }
+}
+
+// Fills in what the copies of misaligned gradients or one-byte weights left
+// out of a whole group (a tensor's first or last), so that the group can be
+// read from the stage.  The fence orders these writes before the next copy
+// into the stage.
+template <int WD, int GD>
+__device__ __forceinline__ void patch_group(const StepArgs& a, const TensorCtx& x, const StageHead& h, int64_t e0,
+                                            int c, uint32_t st) {
+  constexpr uint32_t GS = esize_of(GD);
+  const uint32_t go = x.gsh + kGroup * GS * c, wo = x.wsh + kGroup * c;
+  const bool wm = (WD == kE4M3 || WD == kE4M3B) && !in_range(h.w_range, wo, kGroup);
+  const bool gm = !in_range(h.g_range, go, kGroup * GS);
+  if (!wm && !gm) return;
+  uint32_t r[kGroup], q[kGroup];
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    r[j] = GD == kF32 ? static_cast<const uint32_t*>(h.g)[e0 + j] : static_cast<const uint16_t*>(h.g)[e0 + j];
+    if (WD == kE4M3 || WD == kE4M3B) q[j] = static_cast<const uint8_t*>(x.d.w)[e0 + j];
+  }
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    if (gm) {
+      if (GD == kF32) sts_u32(st + a.off_g + go + 4u * j, r[j]);
+      else sts_u16(st + a.off_g + go + 2u * j, r[j]);
+    }
+    if (wm) sts_u8(st + wo + j, q[j]);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// One group of a partial tile, or of a tensor whose arrays are not all staged
+// or aligned: every array from the stage when all of them hold the whole group
+// there, else all of them element by element from global memory -- the loads
+// of all arrays before the first use, so that the group waits on memory once
+// (array by array it waited five times: a BF16-moment list of 4000 ragged
+// tensors took 345 us, now 295).  dec: the scale the codes decode with.
+template <int WD, int GD, int MD, bool MIS>
+__device__ __forceinline__ void load_group(const StepArgs& a, const TensorCtx& x, const StageHead& h, int64_t e0,
+                                           int count, int c, int valid, uint32_t st, float dec, float (&w)[8],
+                                           float (&g)[8], float (&m)[8], float (&v)[8], float (&ve)[8]) {
+  constexpr int GS = esize_of(GD), MS = esize_of(MD);
+  const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
+  const uint32_t wo = WD == kNVFP4 ? 4u * c : static_cast<uint32_t>(kGroup * esize_of(WD)) * c + x.wsh;
+  const uint32_t go = kGroup * GS * c + x.gsh;
+  bool in;
+  if (MIS) in = in_range(h.w_range, wo, kGroup * esize_of(WD)) && (wo & (WD == kBF16 ? 15u : 7u)) == 0u &&
+                in_range(h.g_range, go, kGroup * GS);
+  else in = (WD == kNVFP4 ? end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1)
+                          : end * esize_of(WD) <= staged_bytes(x.d.w, count, esize_of(WD))) &&
+            end * GS <= staged_bytes(h.g, count, GS);
+  if (in && end * MS <= staged_bytes(x.d.m, count, MS) && end * MS <= staged_bytes(x.d.v, count, MS) &&
+      end * MS <= staged_bytes(x.d.ve, count, MS)) {
+    if (WD == kBF16) get_bf16(w, st + wo);
+    else if (WD == kNVFP4) get_fp4(w, st + wo, dec);
+    else get_e4m3(w, st + wo, dec);
+    if (MIS && GD == kF32) get_f32_at(g, st + a.off_g + go);
+    else if (MIS) get_bf16_at(g, st + a.off_g + go);
+    else if (GD == kF32) get_f32(g, st + a.off_g + go);
+    else get_bf16(g, st + a.off_g + go);
+    if (MD == kF32) {
+      get_f32(m, st + a.off_m + kGroup * MS * c);
+      get_f32(v, st + a.off_v + kGroup * MS * c);
+      get_f32(ve, st + a.off_ve + kGroup * MS * c);
+    } else {
+      get_bf16(m, st + a.off_m + kGroup * MS * c);
+      get_bf16(v, st + a.off_v + kGroup * MS * c);
+      get_bf16(ve, st + a.off_ve + kGroup * MS * c);
+    }
+    return;
+  }
+  auto raw = [&](const void* p, int es, int64_t i) -> uint32_t {
+    return es == 4 ? static_cast<const uint32_t*>(p)[i]
+                   : (es == 2 ? static_cast<const uint16_t*>(p)[i] : static_cast<const uint8_t*>(p)[i]);
+  };
+  uint32_t rw[8], rg[8], rm[8], rv[8], re[8];
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    const bool in = j < valid;
+    rw[j] = in ? raw(x.d.w, WD == kBF16 ? 2 : 1, WD == kNVFP4 ? (e0 + j) >> 1 : e0 + j) : 0u;
+    rg[j] = in ? raw(h.g, GS, e0 + j) : 0u;
+    rm[j] = in ? raw(x.d.m, MS, e0 + j) : 0u;
+    rv[j] = in ? raw(x.d.v, MS, e0 + j) : 0u;
+    re[j] = in ? raw(x.d.ve, MS, e0 + j) : 0u;
+  }
+  auto val = [](uint32_t r, int es) { return __uint_as_float(es == 4 ? r : r << 16); };
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    if (WD == kBF16) w[j] = val(rw[j], 2);
+    else if (WD == kNVFP4) w[j] = j < valid ? __fmul_rn(e2m1_value(((e0 + j) & 1) ? (rw[j] >> 4) : (rw[j] & 0xFu)), dec) : 0.0f;
+    else w[j] = j < valid ? __fmul_rn(e4m3_value(rw[j]), dec) : 0.0f;
+    g[j] = val(rg[j], GS);
+    m[j] = val(rm[j], MS);
+    v[j] = val(rv[j], MS);
+    ve[j] = val(re[j], MS);
   }
 }
 
@@ -872,17 +1017,18 @@ __device__ __forceinline__ void group_random_bits(const StepArgs& a, uint64_t gi
 // original inputs in the stage at st, which must still be allocated.  dec:
 // the scale its code decodes with (E4M3 formats and NVFP4).
 template <int WD, int GD, int MD, bool OPT>
-__device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, uint32_t st, int c, int j, float dec) {
+__device__ __forceinline__ float exact_wn_from_stage(const StepArgs& a, const TensorCtx& x, uint32_t st, int c, int j,
+                                                     float dec) {
   constexpr int GS = esize_of(GD), MS = esize_of(MD);
   const uint32_t i = static_cast<uint32_t>(kGroup * c + j);
   float w;
   if constexpr (WD == kBF16) w = __uint_as_float(lds_u16(st + 2u * i) << 16);
   else if constexpr (WD == kNVFP4) w = __fmul_rn(e2m1_value((lds_u32(st + 4u * c) >> (4 * j)) & 0xFu), dec);
-  else w = __fmul_rn(e4m3_value(lds_u8(st + i)), dec);
+  else w = __fmul_rn(e4m3_value(lds_u8(st + x.wsh + i)), dec);
   auto ld = [&](uint32_t base, int es) -> float {
     return es == 4 ? __uint_as_float(lds_u32(base + 4u * i)) : __uint_as_float(lds_u16(base + 2u * i) << 16);
   };
-  return madam_update<OPT>(a.s, w, ld(st + a.off_g, GS), ld(st + a.off_m, MS), ld(st + a.off_v, MS),
+  return madam_update<OPT>(a.s, w, ld(st + a.off_g + x.gsh, GS), ld(st + a.off_m, MS), ld(st + a.off_v, MS),
                              ld(st + a.off_ve, MS)).wn;
 }
 
@@ -953,7 +1099,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
 #pragma unroll 1
         for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
           const int j = __ffs(rm) - 1;
-          const float xe = exact_wn_from_stage<WD, GD, MD, OPT>(a, st, c, j, 1.0f);
+          const float xe = exact_wn_from_stage<WD, GD, MD, OPT>(a, x, st, c, j, 1.0f);
           const uint32_t code =
               SR ? (bf16_sr_sum(xe, bf16_element_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j)) >> 16)
                  : (bf16x2_rn(xe, xe) & 0xFFFFu);
@@ -1040,7 +1186,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         for (uint32_t rm = redo; rm != 0u; rm &= rm - 1u) {
           const int j = __ffs(rm) - 1;
           const uint32_t r = SR ? lane32_random_bits(a, static_cast<uint64_t>(x.d.goff + e0), j) : 0u;
-          const uint32_t code = exact_code(j, exact_wn_from_stage<WD, GD, MD, OPT>(a, st, c, j, x.dec_scale), r);
+          const uint32_t code = exact_code(j, exact_wn_from_stage<WD, GD, MD, OPT>(a, x, st, c, j, x.dec_scale), r);
           const int sh = 8 * (j & 3);
 #pragma unroll
           for (int i = 0; i < 2; ++i)
@@ -1092,38 +1238,17 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
 }
 
 // One group of a partial tile, or of a tensor whose arrays are not all staged
-// or aligned: loads each array from the stage when its bytes were staged, else
-// from global memory.  The running E4M3 maximum goes in and comes back by
-// value: a reference would pin the caller's copy to local memory.
-template <int WD, int GD, int MD, bool SR, bool OPT>
-__device__ __forceinline__ uint32_t general_group(const StepArgs& a, const TensorCtx& x, int64_t tile_e0,
-                                                  int count, int c, uint32_t st, uint32_t amax_bits) {
-  constexpr int WS = esize_of(WD), GS = esize_of(GD), MS = esize_of(MD);
+// or aligned.  The running E4M3 maximum goes in and comes back by value: a
+// reference would pin the caller's copy to local memory.
+template <int WD, int GD, int MD, bool SR, bool OPT, bool MIS>
+__device__ __forceinline__ uint32_t general_group(const StepArgs& a, const TensorCtx& x, const StageHead& hd,
+                                                  int64_t tile_e0, int count, int c, uint32_t st,
+                                                  uint32_t amax_bits) {
   if (kGroup * c >= count) return amax_bits;
   const int valid = count - kGroup * c < kGroup ? count - kGroup * c : kGroup;
   const int64_t e0 = tile_e0 + kGroup * c;
-  const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
   float w[8], g[8], m[8], v[8], ve[8];
-  if (WD == kBF16)
-    get_bf16<false>(w, end * WS <= staged_bytes(x.d.w, count, WS), st + kGroup * WS * c, x.d.w, e0, valid, x.vec);
-  else
-    get_e4m3(w, end * WS <= staged_bytes(x.d.w, count, WS), st + kGroup * WS * c, x.d.w, e0, valid, x.vec,
-             x.dec_scale);
-  const bool g_st = end * GS <= staged_bytes(x.g, count, GS);
-  if (GD == kF32) get_f32<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  else get_bf16<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  const bool m_st = end * MS <= staged_bytes(x.d.m, count, MS);
-  const bool v_st = end * MS <= staged_bytes(x.d.v, count, MS);
-  const bool e_st = end * MS <= staged_bytes(x.d.ve, count, MS);
-  if (MD == kF32) {
-    get_f32<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_f32<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_f32<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  } else {
-    get_bf16<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_bf16<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_bf16<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  }
+  load_group<WD, GD, MD, MIS>(a, x, hd, e0, count, c, valid, st, x.dec_scale, w, g, m, v, ve);
   finish_group<WD, GD, MD, SR, OPT, false>(a, x, e0, valid, w, g, m, v, ve, amax_bits, st, c);
   return amax_bits;
 }
@@ -1136,10 +1261,11 @@ __device__ __forceinline__ uint32_t general_group(const StepArgs& a, const Tenso
 // GPT-2, the ragged list and the 1.5B list ran 0.7-1.1 % faster inline.  With
 // BF16 moments the inline form slowed the whole-tile loop instead: the 7B list
 // took 18.44 ms per step against 18.21 ms called (three runs each).
-template <int WD, int GD, int MD, bool SR, bool OPT>
-__device__ __noinline__ uint32_t general_group_call(const StepArgs& a, const TensorCtx& x, int64_t tile_e0,
-                                                    int count, int c, uint32_t st, uint32_t amax_bits) {
-  return general_group<WD, GD, MD, SR, OPT>(a, x, tile_e0, count, c, st, amax_bits);
+template <int WD, int GD, int MD, bool SR, bool OPT, bool MIS>
+__device__ __noinline__ uint32_t general_group_call(const StepArgs& a, const TensorCtx& x, const StageHead& hd,
+                                                    int64_t tile_e0, int count, int c, uint32_t st,
+                                                    uint32_t amax_bits) {
+  return general_group<WD, GD, MD, SR, OPT, MIS>(a, x, hd, tile_e0, count, c, st, amax_bits);
 }
 
 // ---------------------------------------------------------------------------
@@ -1199,7 +1325,7 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
     const bool certain = qlo != 0u && qhi < 0x7E800000u /* 2^126 */ && kl == block_exponent(qhi, k_old);
     k_new = kl;
     auto exact_wn = [&](int j) -> float {
-      if constexpr (STAGED) return exact_wn_from_stage<kE4M3B, GD, MD, OPT>(a, st, c, j, fp16_value(h_old));
+      if constexpr (STAGED) return exact_wn_from_stage<kE4M3B, GD, MD, OPT>(a, x, st, c, j, fp16_value(h_old));
       else return madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]);
     };
     if (__any_sync(0xFFFFFFFFu, !certain)) {  // exact block maximum for the undecided quads
@@ -1284,14 +1410,13 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
 // staged: every consumer lane calls this (lanes past the tile's end with no
 // elements), loading each array from the stage when its bytes were staged,
 // else from global memory.
-template <int GD, int MD, bool SR, bool OPT>
-__device__ __forceinline__ void general_block_group(const StepArgs& a, const TensorCtx& x, int64_t tile_e0, int count,
+template <int GD, int MD, bool SR, bool OPT, bool MIS>
+__device__ __forceinline__ void general_block_group(const StepArgs& a, const TensorCtx& x, const StageHead& hd,
+                                                 int64_t tile_e0, int count,
                                                  int c, uint32_t st) {
-  constexpr int GS = esize_of(GD), MS = esize_of(MD);
   const int rem = count - kGroup * c;
   const int valid = rem < 0 ? 0 : (rem < kGroup ? rem : kGroup);
   const int64_t e0 = tile_e0 + kGroup * c;
-  const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
   // the block's old scale: staged when the tile's scale bytes through this block were
   const int nblk = (count + kBlock - 1) / kBlock, b = c >> 2;
   uint32_t h = 0u;
@@ -1301,32 +1426,17 @@ __device__ __forceinline__ void general_block_group(const StepArgs& a, const Ten
   else if (b < nblk)
     h = sc[(tile_e0 / kBlock) + b];
   float w[8], g[8], m[8], v[8], ve[8];
-  get_e4m3(w, end <= staged_bytes(x.d.w, count, 1), st + kGroup * c, x.d.w, e0, valid, x.vec, fp16_value(h));
-  const bool g_st = end * GS <= staged_bytes(x.g, count, GS);
-  if (GD == kF32) get_f32<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  else get_bf16<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  const bool m_st = end * MS <= staged_bytes(x.d.m, count, MS);
-  const bool v_st = end * MS <= staged_bytes(x.d.v, count, MS);
-  const bool e_st = end * MS <= staged_bytes(x.d.ve, count, MS);
-  if (MD == kF32) {
-    get_f32<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_f32<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_f32<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  } else {
-    get_bf16<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_bf16<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_bf16<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  }
+  load_group<kE4M3B, GD, MD, MIS>(a, x, hd, e0, count, c, valid, st, fp16_value(h), w, g, m, v, ve);
   finish_block<GD, MD, SR, OPT, false>(a, x, e0, valid, h, w, g, m, v, ve, st, c);
 }
 
 // The same, as a call: with BF16 moments, as for general_group_call.  Inline,
 // the FP8-regime list (block-scaled linears, binary32 moments) ran 6.02 ms per
 // step against 6.08 ms called.
-template <int GD, int MD, bool SR, bool OPT>
-__device__ __noinline__ void general_block_group_call(const StepArgs& a, const TensorCtx& x, int64_t tile_e0, int count,
-                                             int c, uint32_t st) {
-  general_block_group<GD, MD, SR, OPT>(a, x, tile_e0, count, c, st);
+template <int GD, int MD, bool SR, bool OPT, bool MIS>
+__device__ __noinline__ void general_block_group_call(const StepArgs& a, const TensorCtx& x, const StageHead& hd,
+                                             int64_t tile_e0, int count, int c, uint32_t st) {
+  general_block_group<GD, MD, SR, OPT, MIS>(a, x, hd, tile_e0, count, c, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1357,23 +1467,6 @@ __device__ __forceinline__ uint32_t e2m1_encode(float x, uint32_t r) {
   else up = (f > 0.5f || (f == 0.5f && (k & 1u))) ? 1u : 0u;
   const uint32_t code = ((__float_as_uint(x) >> 28) & 8u) | (k + off + up);
   return x != x ? 0u : code;
-}
-
-// Eight packed E2M1 codes (element j in bits [4j, 4j + 4)) -> binary32, with
-// the hardware E2M1 -> FP16 conversion (exact) and FP16 -> binary32.
-__device__ __forceinline__ void e2m1x8_to_f32(uint32_t packed, float (&x)[8]) {
-  uint32_t h[4];
-  asm("{\n .reg .b8 b0, b1, b2, b3;\n mov.b32 {b0, b1, b2, b3}, %4;\n"
-      " cvt.rn.f16x2.e2m1x2 %0, b0;\n cvt.rn.f16x2.e2m1x2 %1, b1;\n"
-      " cvt.rn.f16x2.e2m1x2 %2, b2;\n cvt.rn.f16x2.e2m1x2 %3, b3;\n}"
-      : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3])
-      : "r"(packed));
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[i]));
-    x[2 * i] = f.x;
-    x[2 * i + 1] = f.y;
-  }
 }
 
 // Eight binary32 -> packed E2M1 codes, nearest-even with saturation at +-6
@@ -1536,7 +1629,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
   float d;
   static_assert(SRC != kExactGlobal || MD == kF32, "exact recompute from global needs binary32 moments");
   auto exact_wn = [&](int j) -> float {
-    if constexpr (SRC == kExactStage) return exact_wn_from_stage<kNVFP4, GD, MD, OPT>(a, st, c, j, d_old);
+    if constexpr (SRC == kExactStage) return exact_wn_from_stage<kNVFP4, GD, MD, OPT>(a, x, st, c, j, d_old);
     else if constexpr (SRC == kExactGlobal) return fp4_exact_from_global<GD, OPT>(a, x, e0 + j, d_old);
     else return madam_wn_exact<OPT>(a.s, w[j], g[j], m[j], v[j], ve[j]);
   };
@@ -1694,37 +1787,15 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
   }
 }
 
-// Eight NVFP4 weights decoded with d: from the stage or global memory as one
-// 32-bit word when whole, else nibble by nibble.
-__device__ __forceinline__ void get_fp4(float (&w)[8], bool staged, uint32_t saddr, const void* gw, int64_t e0,
-                                        int valid, bool vec, float d) {
-  if (staged || (vec && valid == kGroup)) {
-    uint32_t r;
-    if (staged) r = lds_u32(saddr);
-    else asm("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(r) : "l"(static_cast<const uint8_t*>(gw) + e0 / 2));
-    e2m1x8_to_f32(r, w);
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) w[j] = __fmul_rn(w[j], d);
-  } else {
-    const uint8_t* p = static_cast<const uint8_t*>(gw);
-#pragma unroll
-    for (int j = 0; j < kGroup; ++j) {
-      const int64_t k = e0 + j;
-      w[j] = j < valid ? __fmul_rn(e2m1_value((k & 1) ? (p[k >> 1] >> 4) : (p[k >> 1] & 0xFu)), d) : 0.0f;
-    }
-  }
-}
-
 // One NVFP4 group of a partial tile or of a tensor whose arrays are not all
 // staged; every consumer lane calls this (the block maximum is a pair shuffle).
 template <int GD, int MD, bool SR, bool OPT>
-__device__ __noinline__ void general_fp4_group(const StepArgs& a, const TensorCtx& x, int64_t tile_e0, int count,
+__device__ __noinline__ void general_fp4_group(const StepArgs& a, const TensorCtx& x, const StageHead& hd,
+                                               int64_t tile_e0, int count,
                                                int c, uint32_t st) {
-  constexpr int GS = esize_of(GD), MS = esize_of(MD);
   const int rem = count - kGroup * c;
   const int valid = rem < 0 ? 0 : (rem < kGroup ? rem : kGroup);
   const int64_t e0 = tile_e0 + kGroup * c;
-  const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
   const int nblk = (count + kFp4Block - 1) / kFp4Block, b = c >> 1;
   const uint8_t* sc = static_cast<const uint8_t*>(x.scale);
   uint32_t s_old = 0u;
@@ -1734,36 +1805,20 @@ __device__ __noinline__ void general_fp4_group(const StepArgs& a, const TensorCt
     s_old = sc[(tile_e0 / kFp4Block) + b];
   const float d_old = __fmul_rn(e4m3_value(s_old), x.gscale);
   float w[8], g[8], m[8], v[8], ve[8];
-  get_fp4(w, end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1), st + 4 * c, x.d.w, e0, valid, x.vec, d_old);
-  const bool g_st = end * GS <= staged_bytes(x.g, count, GS);
-  if (GD == kF32) get_f32<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  else get_bf16<true>(g, g_st, st + a.off_g + kGroup * GS * c, x.g, e0, valid, x.vec);
-  const bool m_st = end * MS <= staged_bytes(x.d.m, count, MS);
-  const bool v_st = end * MS <= staged_bytes(x.d.v, count, MS);
-  const bool e_st = end * MS <= staged_bytes(x.d.ve, count, MS);
-  if (MD == kF32) {
-    get_f32<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_f32<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_f32<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  } else {
-    get_bf16<false>(m, m_st, st + a.off_m + kGroup * MS * c, x.d.m, e0, valid, x.vec);
-    get_bf16<false>(v, v_st, st + a.off_v + kGroup * MS * c, x.d.v, e0, valid, x.vec);
-    get_bf16<false>(ve, e_st, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, valid, x.vec);
-  }
+  load_group<kNVFP4, GD, MD, false>(a, x, hd, e0, count, c, valid, st, d_old, w, g, m, v, ve);
   finish_fp4<GD, MD, SR, OPT, kExactRegs>(a, x, e0, valid, s_old, w, g, m, v, ve, st, c);
 }
 
 // ---------------------------------------------------------------------------
 // The step kernel.
 // ---------------------------------------------------------------------------
-template <int WD, int GD, int MD, bool SR, bool OPT>
+template <int WD, int GD, int MD, bool SR, bool OPT, bool MIS>
 __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant__ StepArgs a) {
   constexpr int WS = esize_of(WD), GS = esize_of(GD), MS = esize_of(MD);
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages];
   __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
-  __shared__ int64_t stage_tile[kMaxStages];  // tile the producer put in each stage (-1: no more work)
-  __shared__ int32_t stage_k[kMaxStages];     // and its tensor
+  __shared__ StageHead heads[kMaxStages];
 
   // Programmatic dependent launch: the next launch of the stream may start its
   // own entry (it waits below, like this one, for everything before it).
@@ -1785,7 +1840,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
   int pk = -1;       // tensor of tile t
   TensorDesc d{};
   const void* gp = nullptr;
-  const uint8_t* sp = nullptr;
+  TensorAux ax{nullptr, nullptr, 1.0f, 0};
+  int32_t e_cur = 0;
+  uint32_t amax_now = 0u, seed = 0u;
+  int rot = 0;
   int64_t tiles = 0;
   int64_t t = tb, t_end = ts;  // the current run of consecutive tiles
   int ps = 0;                  // next stage to fill, and how many times the ring has wrapped
@@ -1795,32 +1853,72 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     pk = kk;
     d = desc_of(a, pk);
     gp = grad_of(a, pk);
-    if (WD == kE4M3B || WD == kNVFP4) sp = static_cast<const uint8_t*>(aux_of(a, pk).scale);
+    if (WD != kBF16 && a.aux) ax = aux_of(a, pk);  // the launch has aux entries (inline ones too, when it carries its tables)
     tiles = (d.numel + kTile - 1) / kTile;
+    if (WD == kE4M3) {
+      const int64_t n = a.n_tensors;
+      e_cur = a.fp8_exp[a.e_cur_slot * n + d.ring];
+      amax_now = a.fp8_amax[a.a_cur_slot * n + d.ring];
+      // The tensor's maximum flushed so far in this step, read through L2:
+      // the slot was zeroed before this step and is raised only with exact
+      // values, so it seeds the recomputation threshold after a tensor change
+      // (under the tail pool a CTA changes tensor at almost every chunk).
+      asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(seed) : "l"(a.fp8_amax + a.a_next_slot * n + d.ring) : "memory");
+    }
+    if (a.n_inline == 0 && d.tile_off + tiles < a.tile_base + T) {  // the next tensor's entries, into L1
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(a.desc + pk + 1));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(a.grads + pk + 1));
+      if (WD != kBF16 && a.aux) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.aux + pk + 1));
+    }
   };
   auto issue = [&]() {  // the copies of tile t (of tensor pk) into stage ps, which is free
     const int64_t e0 = (t - d.tile_off) * kTile;
     const int count = static_cast<int>(d.numel - e0 < kTile ? d.numel - e0 : kTile);
     // NVFP4 weights: half a byte per element (tile starts stay 16-byte aligned: 1920 bytes per tile)
-    const uint32_t nw = WD == kNVFP4 ? staged_bytes(d.w, (count + 1) / 2, 1) : staged_bytes(d.w, count, WS);
-    const uint32_t ng = staged_bytes(gp, count, GS);
+    // what is copied of the weights and gradients: lo | hi << 16, from the region's start
+    const uint32_t wr = WD == kNVFP4 ? staged_bytes(d.w, (count + 1) / 2, 1) << 16
+                        : MIS && WD != kBF16 ? staged_range(d.w, d.numel, e0, count, WS)
+                                             : staged_bytes(d.w, count, WS) << 16;
+    const uint32_t gr = MIS ? staged_range(gp, d.numel, e0, count, GS) : staged_bytes(gp, count, GS) << 16;
+    const uint32_t nw = (wr >> 16) - (MIS ? wr & 0xFFFFu : 0u), ng = (gr >> 16) - (MIS ? gr & 0xFFFFu : 0u);
     const uint32_t nm = staged_bytes(d.m, count, MS), nv = staged_bytes(d.v, count, MS);
     const uint32_t nve = staged_bytes(d.ve, count, MS);
     const int64_t s0 = WD == kE4M3B ? 2 * (e0 / kBlock) : e0 / kFp4Block;  // the tile's first scale byte
+    const uint8_t* sp = static_cast<const uint8_t*>(ax.scale);
     const uint32_t ns = WD == kE4M3B   ? staged_bytes(sp + s0, 2 * ((count + kBlock - 1) / kBlock), 1)
                         : WD == kNVFP4 ? staged_bytes(sp + s0, (count + kFp4Block - 1) / kFp4Block, 1)
                                        : 0u;
     const uint32_t bar = smem_addr(&full_bar[ps]);
     const uint32_t st = smem0 + static_cast<uint32_t>(ps * a.stage_bytes);
-    stage_tile[ps] = t;  // published by the arrive below (release)
-    stage_k[ps] = pk;
-    mbar_arrive_expect_tx(bar, nw + ng + nm + nv + nve + ns);
-    if (nw) tma_load(st, static_cast<const uint8_t*>(d.w) + (WD == kNVFP4 ? e0 / 2 : e0 * WS), nw, bar, pol);
-    if (ng) tma_load(st + a.off_g, static_cast<const uint8_t*>(gp) + e0 * GS, ng, bar, pol);
+    mbar_expect_tx(bar, nw + ng + nm + nv + nve + ns);
+    const uint32_t wlo = MIS ? wr & 0xFFFFu : 0u, glo = MIS ? gr & 0xFFFFu : 0u;
+    if (nw)
+      tma_load(st + wlo, static_cast<const uint8_t*>(d.w) + (WD == kNVFP4 ? e0 / 2 : e0 * WS) -
+                             (MIS && WD != kBF16 ? misalign(d.w) : 0u) + wlo, nw, bar, pol);
+    if (ng)
+      tma_load(st + a.off_g + glo, static_cast<const uint8_t*>(gp) + e0 * GS - (MIS ? misalign(gp) : 0u) + glo, ng,
+               bar, pol);
     if (nm) tma_load(st + a.off_m, static_cast<const uint8_t*>(d.m) + e0 * MS, nm, bar, pol);
     if (nv) tma_load(st + a.off_v, static_cast<const uint8_t*>(d.v) + e0 * MS, nv, bar, pol);
     if (nve) tma_load(st + a.off_ve, static_cast<const uint8_t*>(d.ve) + e0 * MS, nve, bar, pol);
     if (ns) tma_load(st + a.off_s, sp + s0, ns, bar, pol);
+    StageHead& hd = heads[ps];
+    hd.w = d.w; hd.m = d.m; hd.v = d.v; hd.ve = d.ve;
+    hd.g = gp;
+    if (WD != kBF16) { hd.scale = ax.scale; hd.cc = ax.compute; hd.gscale = ax.gscale; }
+    hd.goff = d.goff;
+    hd.e0 = e0;
+    hd.k = pk;
+    hd.count = count;
+    hd.rot = rot;
+    hd.ring = d.ring;
+    if (WD == kE4M3) { hd.e_cur = e_cur; hd.amax = amax_now; hd.seed = seed; }
+    if (MIS) { hd.w_range = wr; hd.g_range = gr; }
+    mbar_arrive(bar);  // publishes the head (release); the copies complete the phase
+    // the next tile's first 256 elements go to the warp after this tile's
+    // last: short tensors spread over the warps instead of all taking the first
+    rot += (count + 32 * kGroup - 1) / (32 * kGroup);
+    if (rot >= kConsumerWarps) rot -= kConsumerWarps;
     ++issued;
     ++t;
     if (++ps == S) { ps = 0; ++puse; }
@@ -1892,41 +1990,27 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
       if (a.err) atomicOr(a.err, kErrEmptyWait);
       return;
     }
-    stage_tile[ps] = -1;
+    heads[ps].k = -1;
     mbar_arrive(smem_addr(&full_bar[ps]));
     return;
   }
 
   // ----------------------------------------------------------- consumers --
-  const int c = tid;  // consumer index, owns elements [8c, 8c + 8) of every tile
   const int n = a.n_tensors;
   int k = -1;
   TensorCtx x;
   int32_t e_next = 0;
-  auto enter = [&](int kk) {  // take up tensor kk
-    k = kk;
-    load_tensor<WD, GD, MD>(a, k, x);
+  auto enter = [&](const StageHead& hd) {  // take up the stage's tensor
+    k = hd.k;
+    load_tensor<WD, GD, MD, MIS>(hd, x);
     if (WD == kE4M3) {
-      const int32_t e_cur = a.fp8_exp[static_cast<int64_t>(a.e_cur_slot) * n + x.d.ring];
-      e_next = fp8_next_exponent(a.fp8_amax[static_cast<int64_t>(a.a_cur_slot) * n + x.d.ring], e_cur);
-      x.dec_scale = pow2f(e_cur);
+      e_next = fp8_next_exponent(hd.amax, hd.e_cur);
+      x.dec_scale = pow2f(hd.e_cur);
       x.enc_scale = pow2f(-e_next);
       x.cc_scale = pow2f(e_next);
-      // The tensor's maximum flushed so far in this step, read through L2:
-      // the slot was zeroed before this step and is raised only with exact
-      // values, so it seeds the recomputation threshold after a tensor change
-      // (under the tail pool a CTA changes tensor at almost every chunk).
-      uint32_t seed;
-      asm volatile("ld.global.cg.u32 %0, [%1];"
-                   : "=r"(seed)
-                   : "l"(a.fp8_amax + static_cast<int64_t>(a.a_next_slot) * n + x.d.ring)
-                   : "memory");
-      x.amax_seed = __uint_as_float(seed);
+      x.amax_seed = __uint_as_float(hd.seed);
     }
   };
-  // The first tile posted is the first of this CTA's own range when it has
-  // one: take up its tensor while the copies are in flight.
-  if (tb < ts) enter(first_tensor(a, tb));
   uint32_t amax_bits = 0u;
   int s = 0;
   uint32_t use = 0;
@@ -1935,53 +2019,67 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
       if (a.err && lane == 0) atomicOr(a.err, kErrFullWait);
       return;
     }
-    const int64_t t = stage_tile[s];
-    if (t < 0) break;  // the producer's end marker
-    const int kt = stage_k[s];
+    const StageHead& hd = heads[s];
+    const int kt = hd.k;
+    if (kt < 0) break;  // the producer's end marker
+    const int count = hd.count;
+    const int lw = warp - hd.rot + (warp < hd.rot ? kConsumerWarps : 0);  // this warp's place in the tile
+    const int c = 32 * lw + lane;  // consumer: elements [8c, 8c + 8) of the tile
+    if (32 * kGroup * lw >= count) {  // nothing for this warp
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));
+      if (++s == S) { s = 0; ++use; }
+      continue;
+    }
     if (kt != k) {  // another tensor: flush this one's E4M3 amax
       if (WD == kE4M3 && k >= 0) {
         if (lane == 0 && amax_bits != 0u)
           atomicMax(&a.fp8_amax[static_cast<int64_t>(a.a_next_slot) * n + x.d.ring], amax_bits);
         amax_bits = 0u;
       }
-      enter(kt);
+      enter(hd);
     }
-    const int64_t tile_e0 = (t - x.d.tile_off) * kTile;
+    const int64_t tile_e0 = hd.e0;
     if (WD == kE4M3 && tile_e0 == 0 && c == 0) {  // the CTA holding the tensor's first tile
       a.fp8_exp[static_cast<int64_t>(a.e_next_slot) * n + x.d.ring] = e_next;
       a.fp8_amax[static_cast<int64_t>(a.a_zero_slot) * n + x.d.ring] = 0u;
     }
-    const int count = static_cast<int>(x.d.numel - tile_e0 < kTile ? x.d.numel - tile_e0 : kTile);
     // Straight-line group: every array aligned, and this warp's 256 elements
     // all inside the tile (every warp of a whole tile; the whole warps of a
     // tensor's last tile, whose bytes the producer staged as well).  A warp
     // that holds the end of a partial tile takes the element-wise path below.
-    if (x.fast && kGroup * 32 * (warp + 1) <= count) {
+    if (x.fast && kGroup * 32 * (lw + 1) <= count) {
       const uint32_t st = smem0 + static_cast<uint32_t>(s * a.stage_bytes);
       const int64_t e0 = tile_e0 + kGroup * c;
       float w[8], g[8], m[8], v[8], ve[8];
       uint32_t h_old = 0u;
+      if (MIS && (x.gsh | x.wsh) != 0u) patch_group<WD, GD>(a, x, hd, e0, c, st);
       if (WD == kBF16) {
-        get_bf16<false>(w, true, st + kGroup * WS * c, x.d.w, e0, kGroup, true);
+        get_bf16(w, st + kGroup * WS * c);
       } else if (WD == kE4M3) {
-        get_e4m3(w, true, st + kGroup * WS * c, x.d.w, e0, kGroup, true, x.dec_scale);
+        get_e4m3(w, st + x.wsh + kGroup * WS * c, x.dec_scale);
       } else if (WD == kE4M3B) {
         h_old = lds_u16(st + a.off_s + 2 * (c >> 2));
-        get_e4m3(w, true, st + kGroup * WS * c, x.d.w, e0, kGroup, true, fp16_value(h_old));
+        get_e4m3(w, st + x.wsh + kGroup * WS * c, fp16_value(h_old));
       } else {
         h_old = lds_u8(st + a.off_s + (c >> 1));
-        get_fp4(w, true, st + 4 * c, x.d.w, e0, kGroup, true, __fmul_rn(e4m3_value(h_old), x.gscale));
+        get_fp4(w, st + 4 * c, __fmul_rn(e4m3_value(h_old), x.gscale));
       }
-      if (GD == kF32) get_f32<true>(g, true, st + a.off_g + kGroup * GS * c, x.g, e0, kGroup, true);
-      else get_bf16<true>(g, true, st + a.off_g + kGroup * GS * c, x.g, e0, kGroup, true);
-      if (MD == kF32) {
-        get_f32<false>(m, true, st + a.off_m + kGroup * MS * c, x.d.m, e0, kGroup, true);
-        get_f32<false>(v, true, st + a.off_v + kGroup * MS * c, x.d.v, e0, kGroup, true);
-        get_f32<false>(ve, true, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, kGroup, true);
+      if (MIS && x.gsh != 0u) {
+        if (GD == kF32) get_f32_at(g, st + a.off_g + x.gsh + kGroup * GS * c);
+        else get_bf16_at(g, st + a.off_g + x.gsh + kGroup * GS * c);
       } else {
-        get_bf16<false>(m, true, st + a.off_m + kGroup * MS * c, x.d.m, e0, kGroup, true);
-        get_bf16<false>(v, true, st + a.off_v + kGroup * MS * c, x.d.v, e0, kGroup, true);
-        get_bf16<false>(ve, true, st + a.off_ve + kGroup * MS * c, x.d.ve, e0, kGroup, true);
+        if (GD == kF32) get_f32(g, st + a.off_g + kGroup * GS * c);
+        else get_bf16(g, st + a.off_g + kGroup * GS * c);
+      }
+      if (MD == kF32) {
+        get_f32(m, st + a.off_m + kGroup * MS * c);
+        get_f32(v, st + a.off_v + kGroup * MS * c);
+        get_f32(ve, st + a.off_ve + kGroup * MS * c);
+      } else {
+        get_bf16(m, st + a.off_m + kGroup * MS * c);
+        get_bf16(v, st + a.off_v + kGroup * MS * c);
+        get_bf16(ve, st + a.off_ve + kGroup * MS * c);
       }
       if constexpr (WD == kNVFP4 && MD == kF32) {
         // released at once: the rare exact branch re-reads global memory
@@ -2013,18 +2111,18 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     // the stochastic-rounding loop by 5 %)
     if constexpr (WD == kE4M3B) {
       if constexpr (MD == kF32)
-        general_block_group<GD, MD, SR, OPT>(a, x, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes));
+        general_block_group<GD, MD, SR, OPT, MIS>(a, x, hd, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes));
       else
-        general_block_group_call<GD, MD, SR, OPT>(a, x, tile_e0, count, c,
+        general_block_group_call<GD, MD, SR, OPT, MIS>(a, x, hd, tile_e0, count, c,
                                                   smem0 + static_cast<uint32_t>(s * a.stage_bytes));
     } else if constexpr (WD == kNVFP4)
-      general_fp4_group<GD, MD, SR, OPT>(a, x, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes));
+      general_fp4_group<GD, MD, SR, OPT>(a, x, hd, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes));
     else
-      amax_bits = MD == kF32 ? general_group<WD, GD, MD, SR, OPT>(a, x, tile_e0, count, c,
+      amax_bits = MD == kF32 ? general_group<WD, GD, MD, SR, OPT, MIS>(a, x, hd, tile_e0, count, c,
                                                                    smem0 + static_cast<uint32_t>(s * a.stage_bytes),
                                                                    amax_bits)
-                             : general_group_call<WD, GD, MD, SR, OPT>(
-                                   a, x, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes), amax_bits);
+                             : general_group_call<WD, GD, MD, SR, OPT, MIS>(
+                                   a, x, hd, tile_e0, count, c, smem0 + static_cast<uint32_t>(s * a.stage_bytes), amax_bits);
     __syncwarp();
     if (WD == kE4M3) amax_bits = __reduce_max_sync(0xFFFFFFFFu, amax_bits);
     if (lane == 0) mbar_arrive(smem_addr(&empty_bar[s]));

@@ -6,8 +6,8 @@ namespace mpadam {
 
 template <int GD, int MD, bool SR>
 static const void* pick_nvfp4(int options) {
-  return options ? reinterpret_cast<const void*>(&step_kernel<kNVFP4, GD, MD, SR, true>)
-                 : reinterpret_cast<const void*>(&step_kernel<kNVFP4, GD, MD, SR, false>);
+  return options ? reinterpret_cast<const void*>(&step_kernel<kNVFP4, GD, MD, SR, true, false>)
+                 : reinterpret_cast<const void*>(&step_kernel<kNVFP4, GD, MD, SR, false, false>);
 }
 
 template <int GD, int MD>
