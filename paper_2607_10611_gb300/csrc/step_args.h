@@ -141,7 +141,12 @@ struct StepArgs {
   int32_t* err;              // DeviceError bits, or nullptr
   const PoolChunk* pool;     // [pool_chunks] tail pool, or nullptr (static ranges only)
   uint32_t* pool_next;       // next unclaimed pool chunk; zero when the launch starts and again when it ends
-  int32_t pool_chunks;
+  int32_t pool_chunks;       // 0: no pool
+  // A pool without a table (pool == nullptr; the allocation-free step): the
+  // static ranges share tiles [tile_base, pool_base), and chunk j is the
+  // pool_len tiles from pool_base + j pool_len on.
+  int64_t pool_base;
+  int32_t pool_len;          // 0: not this kind
   // Launches of at most kInlineTensors tensors (a flat parameter buffer, a
   // short list) carry their descriptors, aux entries and gradient pointers
   // here as well, so that a CTA finds its first tensor and issues its first

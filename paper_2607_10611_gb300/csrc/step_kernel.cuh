@@ -790,6 +790,18 @@ __device__ __forceinline__ int first_tensor(const StepArgs& a, int64_t tb) {
   return k;
 }
 
+// The tensor holding tile t, at or after tensor k (which starts at or before
+// it): the last one that starts at or before t, by doubling steps and halving
+// ones.  (Empty tensors start where the next one does and come before it.)
+__device__ __forceinline__ int tensor_of(const StepArgs& a, int k, int64_t t) {
+  auto starts = [&](int i) { return i < a.n_tensors && desc_of(a, i).tile_off <= t; };
+  int step = 1;
+  while (starts(k + step)) { k += step; step <<= 1; }
+  for (; step > 0; step >>= 1)
+    if (starts(k + step)) k += step;
+  return k;
+}
+
 // What the producer posts beside each stage: the tile, and everything the
 // consumers need of its tensor.  The producer's loads of the tables run ahead
 // by the depth of the ring; with the consumers loading them at every change of
@@ -1827,9 +1839,11 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
   const int warp = tid >> 5, lane = tid & 31;
   const int S = a.stages;
   const int64_t T = a.total_tiles;
-  const int64_t tb = a.tile_base + static_cast<int64_t>(blockIdx.x) * T / gridDim.x;
-  const int64_t te = a.tile_base + (static_cast<int64_t>(blockIdx.x) + 1) * T / gridDim.x;
-  if (tb >= te && !a.pool) return;
+  const bool pooled = a.pool_chunks > 0;
+  const int64_t split = a.pool_len > 0 ? a.pool_base - a.tile_base : T;  // tiles dealt out to the CTAs' ranges
+  const int64_t tb = a.tile_base + static_cast<int64_t>(blockIdx.x) * split / gridDim.x;
+  const int64_t te = a.tile_base + (static_cast<int64_t>(blockIdx.x) + 1) * split / gridDim.x;
+  if (tb >= te && !pooled) return;
   // static part of the range; the rest went to the tail pool
   const int64_t ts = a.pool ? tb + (te - tb) * a.static_q / 1024 : te;
   const uint32_t smem0 = smem_addr(smem);
@@ -1958,13 +1972,21 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     bool failed = false;
     for (;;) {
       if (t >= t_end) {  // static part done: next chunk of the tail pool, if any
-        if (!a.pool) break;
+        if (!pooled) break;
         const uint32_t j = claim();
         if (j >= static_cast<uint32_t>(a.pool_chunks)) break;
-        const PoolChunk pc = a.pool[j];
-        t = pc.start;
-        t_end = pc.start + pc.count;
-        if (pc.first != pk) load(pc.first);
+        int first;
+        if (a.pool) {
+          const PoolChunk pc = a.pool[j];
+          t = pc.start;
+          t_end = pc.start + pc.count;
+          first = pc.first;
+        } else {  // a pool without a table: the last tiles of the list, pool_len at a time
+          t = a.pool_base + static_cast<int64_t>(j) * a.pool_len;
+          t_end = t + a.pool_len < a.tile_base + T ? t + a.pool_len : a.tile_base + T;
+          first = tensor_of(a, pk < 0 ? 0 : pk, t);
+        }
+        if (first != pk) load(first);
       }
       while (t >= d.tile_off + tiles) load(pk + 1);
       if (puse > 0 && !mbar_wait(smem_addr(&empty_bar[ps]), (puse - 1) & 1u)) {
@@ -1981,7 +2003,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         if (!mbar_wait(smem_addr(&full_bar[it % S]), static_cast<uint32_t>((it / S) & 1)) && a.err)
           atomicOr(a.err, kErrDrainWait);
       }
-      if (a.pool)
+      if (pooled)
         while (claim() < static_cast<uint32_t>(a.pool_chunks)) {}  // leave the counter as a CTA that finished would
       return;
     }
