@@ -233,9 +233,7 @@ int32_t mpadam_fp8_init(mpadam_state* s, const int32_t* init_exp, int64_t first_
  * grads: host array of n device pointers, grads[k] holding numel[k]
  * gradients of grad_dtype (read only).  The pointer table is re-uploaded
  * only when it differs from the previous call's.  On `stream` the call puts
- * one kernel launch per weight format and, while a tail pool is on (see
- * mpadam_set_tail_pool), one cudaMemsetAsync of the pool's counters before
- * them.  Steps of one state must not overlap on the GPU.  The same (inputs, t, seed) reproduce the
+ * one kernel launch per weight format.  Steps of one state must not overlap on the GPU.  The same (inputs, t, seed) reproduce the
  * same bits, so a resumed run calls with the step it stopped at.
  * Errors: EINVAL (t < 1, NULL/misaligned grads), ECUDA (launch). */
 int32_t mpadam_step(mpadam_state* s, const void* const* grads, int64_t step,
@@ -323,12 +321,12 @@ int32_t mpadam_launch_info(const mpadam_state* s, int32_t* ctas, int32_t* thread
  * chunk_tiles tiles, which the CTAs that finish first claim one at a time.
  * SMs do not all stream memory at the same rate, so without the pool a
  * launch waits on the slowest.  static_q = 1024 turns the pool off.
- * Default: static_q = 768, chunk_tiles = 4, for every weight format, except
- * that until this is called a format group with fewer than 8 tiles per CTA
- * keeps static runs (with a tile or two per CTA the pool's first claimants
- * would take several chunks each).  Results do not depend on any of this.
- * Synchronises the device.  The host-buffer and allocation-free entry
- * points always use static runs.
+ * Until this is called the library chooses by tiles per CTA: fewer than 8
+ * keep static runs (with a tile or two per CTA the pool's first claimants
+ * would take several chunks each), then 768 and 4 below 16, 256 and 1 below
+ * 128, and 0 and 2 above (0 and 1 for binary32 moments and long tensors).  Results do not depend on any of this.
+ * Synchronises the device.  The host-buffer entry point always uses static
+ * runs; the allocation-free one chooses as above.
  * Errors: EINVAL (static_q outside [0, 1024], chunk_tiles outside
  * [1, 2^20]), EALLOC, ECUDA. */
 int32_t mpadam_set_tail_pool(mpadam_state* s, int32_t static_q, int32_t chunk_tiles);

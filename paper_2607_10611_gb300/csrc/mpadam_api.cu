@@ -323,6 +323,7 @@ struct Group {
   int32_t cta_cap = 0;
   mpadam::PoolChunk* d_pool = nullptr;  // tail pool of the current grid (none when static_q is 1024)
   int32_t pool_chunks = 0, pool_cap = 0;
+  int32_t static_q = 1024, pool_len = 0;  // static share (1/1024); tiles per chunk of a pool without a table
   std::vector<TensorDesc> h_desc;       // host copies of its table entries (inline in short launches)
   std::vector<TensorAux> h_aux;
 };
@@ -358,8 +359,7 @@ struct mpadam_state {
   std::vector<int64_t> chunk_elem;            // and global elements [chunk_elem[2c], chunk_elem[2c+1])
   int32_t* d_chunk_first = nullptr;           // [chunks][grid] CTA start tensors
   // tail pool of mpadam_step's launches: static prefix of each CTA's range (1/1024) and chunk length;
-  // until set_tail_pool is called, groups of fewer than kPoolMinTilesPerCta tiles per CTA keep
-  // static runs (with a tile or two per CTA, greedy claims would pile chunks on a few CTAs)
+  // as set by set_tail_pool (until then: pool_rule)
   int32_t pool_q = 768, pool_chunk = 4;
   bool pool_set = false;
   uint32_t* d_pool_next = nullptr;            // [groups] claim counters, zero between launches
@@ -483,17 +483,61 @@ int32_t upload_pool(Group& g, int32_t grid, int32_t q, int32_t chunk) {
   return MPADAM_OK;
 }
 
-// The static share a group's launches use: every format (per-tensor E4M3
-// too, whose consumers seed the exact-maximum threshold from the amax ring
-// after each tensor change), but by default only groups with at least
-// kPoolMinTilesPerCta tiles per CTA.  A producer claims chunks while its ring
-// has free stages, so with a tile or two per CTA the first CTAs to reach the
-// pool take several chunks each and the launch waits on them (measured on a
-// 1 Mi-element list: 16.2 us pooled, 14.5 us static).
-constexpr int64_t kPoolMinTilesPerCta = 8;
-int32_t pool_q_of(const mpadam_state* s, const Group& g) {
-  if (!s->pool_set && g.tiles < kPoolMinTilesPerCta * g.grid) return 1024;
-  return s->pool_q;
+// How a launch deals out its tiles, by tiles per CTA.  SMs stream at different
+// rates, so all but the shortest launches take part of their tiles from a pool,
+// in chunks; small chunks even out the end, and with every tile in the pool the
+// SMs walk the list together, which the memory system likes better than 152
+// streams apart (GPT-2 546.4 -> 535.0 us per step, the 1.5B E4M3 list 5452 ->
+// 5399, 100 M in BF16 271.3 -> 263.7).  Measured, static share / chunk:
+//   < 8     all static: with a tile or two per CTA the first CTAs to reach a
+//           pool take several chunks each and the launch waits on them (1 Mi
+//           parameters 16.2 us pooled, 14.5 static);
+//   < 16    3/4, 4 tiles: finer chunks gain with binary32 moments (7 M
+//           parameters 32.3 -> 31.1 us) and lose with BF16 (22.0 -> 23.1);
+//   < 128   1/4, 1 tile (10 M 50.6 -> 48.2 us, BF16 moments 33.3 -> 30.9; 40 M
+//           181.3 -> 176.8, 114.5 -> 109.8);
+//   more    none, 2 tiles; 1 with binary32 moments and no table (GPT-2 530.7
+//           us against 535.0, FP8 regime 2332 against 2351).  Where a tile has
+//           few bytes, or tensors are short, claims of 1 outrun the producers
+//           (a billion in BF16 2794 us with 2, 3064 with 1; 4000 ragged tensors
+//           380 and 388).
+// With none static a chunk's place follows from its number, so a list whose
+// tensors average kPoolSearchTiles tiles or more needs no table: the claimer
+// finds the tensor by search from the one it has (a few steps).
+constexpr int64_t kPoolMinTilesPerCta = 8, kPoolFineTilesPerCta = 16, kPoolAllTilesPerCta = 128;
+constexpr int64_t kPoolSearchTiles = 64;
+
+struct PoolRule {
+  int32_t static_q = 1024, chunk = 4;  // static share in 1/1024 (1024: no pool), tiles per chunk
+  bool search = false;                 // no table (static_q 0)
+};
+
+PoolRule pool_rule(int64_t tiles, int32_t tensors, int32_t grid, int32_t moment_dtype) {
+  PoolRule r;
+  if (tiles < kPoolMinTilesPerCta * grid || tiles >= INT32_MAX) return r;
+  if (tiles < kPoolFineTilesPerCta * grid) {
+    r.static_q = 768;
+  } else if (tiles < kPoolAllTilesPerCta * grid) {
+    r.static_q = 256;
+    r.chunk = 1;
+  } else {
+    r.static_q = 0;
+    r.search = tiles >= kPoolSearchTiles * tensors;
+    r.chunk = r.search && moment_dtype == MPADAM_F32 ? 1 : 2;
+  }
+  return r;
+}
+
+// The group's pool for its grid: as set by the caller, else by the rule.
+int32_t setup_pool(mpadam_state* s, Group& g) {
+  PoolRule r = pool_rule(g.tiles, g.count, g.grid, s->cfg.moment_dtype);
+  if (s->pool_set) r = PoolRule{s->pool_q, s->pool_chunk, false};
+  g.static_q = r.static_q;
+  g.pool_len = 0;
+  if (!r.search) return upload_pool(g, g.grid, r.static_q, r.chunk);
+  g.pool_len = r.chunk;
+  g.pool_chunks = (int32_t)((g.tiles + r.chunk - 1) / r.chunk);
+  return MPADAM_OK;
 }
 
 void fill_common(StepArgs& a, const mpadam_config& cfg, const Geometry& geo, int64_t total_tiles, int32_t n,
@@ -530,6 +574,7 @@ StepArgs base_args(const mpadam_state* s, const Group& g) {
   StepArgs a;
   fill_common(a, s->cfg, g.geo, g.tiles, s->n, s->fp8_exp, s->fp8_amax);
   a.desc = s->d_desc + g.first;
+  a.n_desc = g.count;
   a.aux = g.aux ? s->d_aux + g.first : nullptr;
   a.grads = s->d_grads + g.first;
   a.cta_first = g.d_cta_first;
@@ -714,7 +759,7 @@ int32_t create_state(const std::vector<TensorIn>& t, const mpadam_config* cfg, i
     }
     for (auto& g : s->groups) {
       rc = upload_cta_table(g, g.default_grid);
-      if (!rc) rc = upload_pool(g, g.grid, pool_q_of(s, g), s->pool_chunk);
+      if (!rc) rc = setup_pool(s, g);
       if (rc) { release(s); return rc; }
     }
   } catch (const std::bad_alloc&) {
@@ -775,10 +820,11 @@ int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t 
   a.tile_base = tile_base;
   a.total_tiles = count;
   if (pool_next && g.pool_chunks > 0) {  // whole-group launches only: the pool covers all of its tiles
-    a.pool = g.d_pool;
     a.pool_next = pool_next;
     a.pool_chunks = g.pool_chunks;
-    a.static_q = pool_q_of(s, g);
+    a.static_q = g.static_q;
+    if (g.pool_len > 0) a.pool_len = g.pool_len;  // pool_base 0: every tile is in the pool
+    else a.pool = g.d_pool;
   }
   if (tile_base == 0 && count == g.tiles && g.count <= mpadam::kInlineTensors) {
     // a short whole-group launch carries its tables (the gradient pointers as
@@ -927,7 +973,7 @@ int32_t mpadam_set_grid(mpadam_state* s, int32_t ctas) {
   release_pipeline(s);  // the host-buffer pipeline's per-chunk tables follow the grid: rebuilt on next use
   for (auto& g : s->groups) {
     rc = upload_cta_table(g, ctas == 0 ? g.default_grid : ctas);
-    if (!rc) rc = upload_pool(g, g.grid, pool_q_of(s, g), s->pool_chunk);
+    if (!rc) rc = setup_pool(s, g);
     if (rc) return rc;
   }
   return MPADAM_OK;
@@ -945,7 +991,7 @@ int32_t mpadam_set_tail_pool(mpadam_state* s, int32_t static_q, int32_t chunk_ti
   s->pool_chunk = chunk_tiles;
   s->pool_set = true;
   for (auto& g : s->groups) {
-    rc = upload_pool(g, g.grid, pool_q_of(s, g), s->pool_chunk);
+    rc = setup_pool(s, g);
     if (rc) return rc;
   }
   return MPADAM_OK;
@@ -1310,18 +1356,21 @@ extern "C" int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, 
 
   StepArgs a;
   fill_common(a, *cfg, geo, total_tiles, n, fp8_exp, fp8_amax);
-  // Lists of kPoolMinTilesPerCta tiles per CTA or more leave a quarter to a
-  // pool, as mpadam_step does, with chunks of 4 tiles taken from the end of
-  // the list so that no table is needed (465 M parameters in BF16: 1407 us per
-  // step with static ranges, 1237 with the pool).
+  // The same shares and chunks as mpadam_step's (pool_rule), the pool being the
+  // last tiles of the list so that no table is needed; where tensors are short
+  // (a search per chunk would cost more) a quarter, 4 tiles at a time (465 M
+  // parameters in BF16: 1407 us per step with static ranges, 1208 with the pool).
   int64_t split = total_tiles;
-  if (total_tiles >= kPoolMinTilesPerCta * grid && total_tiles < INT32_MAX) {
-    split = total_tiles * 768 / 1024;
+  PoolRule rule = pool_rule(total_tiles, n, grid, cfg->moment_dtype);
+  if (rule.static_q < 1024) {
+    if (total_tiles < kPoolSearchTiles * n) rule = PoolRule{768, 4, true};
+    split = total_tiles * rule.static_q / 1024;
     a.pool_base = split;
-    a.pool_len = 4;
+    a.pool_len = rule.chunk;
     a.pool_chunks = (int32_t)((total_tiles - split + a.pool_len - 1) / a.pool_len);
     a.pool_next = reinterpret_cast<uint32_t*>(scratch + kNoAllocPoolOffset);
   }
+  a.n_desc = n;
 
   if (n <= mpadam::kInlineTensors) {  // a short list's tables travel with the launch
     int64_t off = 0, toff = 0;

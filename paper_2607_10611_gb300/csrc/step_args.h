@@ -124,6 +124,7 @@ struct StepArgs {
   int64_t tile_base;         // this launch covers tiles [tile_base, tile_base + total_tiles)
   int64_t total_tiles;
   int32_t n_tensors;         // length of the whole list (stride of the scale rings)
+  int32_t n_desc;            // descriptors of this launch
   int32_t stages;            // shared-memory pipeline depth (2..kMaxStages)
   int32_t stage_bytes;       // bytes of one stage: w | g | m | v | ve | block-scale regions
   int32_t off_g, off_m, off_v, off_ve;  // region offsets inside a stage (w at 0)
@@ -142,9 +143,8 @@ struct StepArgs {
   const PoolChunk* pool;     // [pool_chunks] tail pool, or nullptr (static ranges only)
   uint32_t* pool_next;       // next unclaimed pool chunk; zero when the launch starts and again when it ends
   int32_t pool_chunks;       // 0: no pool
-  // A pool without a table (pool == nullptr; the allocation-free step): the
-  // static ranges share tiles [tile_base, pool_base), and chunk j is the
-  // pool_len tiles from pool_base + j pool_len on.
+  // A pool without a table (pool == nullptr): the static ranges share tiles
+  // [tile_base, pool_base), and chunk j is the pool_len tiles from pool_base + j pool_len on.
   int64_t pool_base;
   int32_t pool_len;          // 0: not this kind
   // Launches of at most kInlineTensors tensors (a flat parameter buffer, a

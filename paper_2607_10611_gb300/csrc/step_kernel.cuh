@@ -794,7 +794,7 @@ __device__ __forceinline__ int first_tensor(const StepArgs& a, int64_t tb) {
 // it): the last one that starts at or before t, by doubling steps and halving
 // ones.  (Empty tensors start where the next one does and come before it.)
 __device__ __forceinline__ int tensor_of(const StepArgs& a, int k, int64_t t) {
-  auto starts = [&](int i) { return i < a.n_tensors && desc_of(a, i).tile_off <= t; };
+  auto starts = [&](int i) { return i < a.n_desc && desc_of(a, i).tile_off <= t; };
   int step = 1;
   while (starts(k + step)) { k += step; step <<= 1; }
   for (; step > 0; step >>= 1)
@@ -1970,10 +1970,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     // (a memset before every launch cost a gap of its own on the stream).
     auto claim = [&]() { return atomicInc(a.pool_next, static_cast<uint32_t>(a.pool_chunks) + gridDim.x - 1u); };
     bool failed = false;
+    bool ahead = false;  // a claim (j) made before the run in hand is done
+    uint32_t j = 0u;
     for (;;) {
       if (t >= t_end) {  // static part done: next chunk of the tail pool, if any
         if (!pooled) break;
-        const uint32_t j = claim();
+        if (!ahead) j = claim();
+        ahead = false;
         if (j >= static_cast<uint32_t>(a.pool_chunks)) break;
         int first;
         if (a.pool) {
@@ -1989,6 +1992,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         if (first != pk) load(first);
       }
       while (t >= d.tile_off + tiles) load(pk + 1);
+      if (pooled && !ahead && t + 1 >= t_end) {  // the run's last tile: its wait for a free stage covers the claim's
+        j = claim();
+        ahead = true;
+      }
       if (puse > 0 && !mbar_wait(smem_addr(&empty_bar[ps]), (puse - 1) & 1u)) {
         if (a.err) atomicOr(a.err, kErrEmptyWait);
         failed = true;
@@ -2003,7 +2010,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         if (!mbar_wait(smem_addr(&full_bar[it % S]), static_cast<uint32_t>((it / S) & 1)) && a.err)
           atomicOr(a.err, kErrDrainWait);
       }
-      if (pooled)
+      if (pooled && !(ahead && j >= static_cast<uint32_t>(a.pool_chunks)))
         while (claim() < static_cast<uint32_t>(a.pool_chunks)) {}  // leave the counter as a CTA that finished would
       return;
     }
