@@ -503,9 +503,11 @@ int32_t upload_pool(Group& g, int32_t grid, int32_t q, int32_t chunk) {
 //           380 and 388).
 // With none static a chunk's place follows from its number, so a list whose
 // tensors average kPoolSearchTiles tiles or more needs no table: the claimer
-// finds the tensor by search from the one it has (a few steps).
+// finds the tensor by search from the one it has (a few steps; 20,000 tensors
+// of 71 tiles on average, most of them short: 23.9 ms by search, 22.9 with the
+// table, 23.5 with 3/4 static).
 constexpr int64_t kPoolMinTilesPerCta = 8, kPoolFineTilesPerCta = 16, kPoolAllTilesPerCta = 128;
-constexpr int64_t kPoolSearchTiles = 64;
+constexpr int64_t kPoolSearchTiles = 128;
 
 struct PoolRule {
   int32_t static_q = 1024, chunk = 4;  // static share in 1/1024 (1024: no pool), tiles per chunk

@@ -500,6 +500,16 @@ cudaError_t launch_toy_run(const ToyArgs& a, int64_t first, int64_t steps, doubl
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&toy_run_kernel),
                                     dim3(static_cast<unsigned>(a.batch / C)), dim3(static_cast<unsigned>(C)), params, 0,
                                     stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs than CTAs to this process: step by step
+      cudaGetLastError();
+      for (int64_t i = 0; i < n; ++i) {
+        args.loss_out = l ? l + i : nullptr;
+        args.t_lo = static_cast<uint32_t>(static_cast<uint64_t>(f + i));
+        args.t_hi = static_cast<uint32_t>(static_cast<uint64_t>(f + i) >> 32);
+        if ((e = launch_toy_step(args, stream)) != cudaSuccess) return e;
+      }
+      continue;
+    }
     if (e != cudaSuccess) return e;
     if (l && a.split) {
       toy_add_losses_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(l, a.loss_hi, n);

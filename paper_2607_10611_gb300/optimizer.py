@@ -25,6 +25,8 @@ _SCALES = {"e4m3_b32": torch.float16, "nvfp4": torch.uint8}
 
 def _pointers(tensors) -> array.array:
     """Device pointers of tensors, as the array that the C ABI takes."""
+    if not isinstance(tensors, (list, tuple)):
+        tensors = list(tensors)
     try:
         return array.array("Q", map(torch.Tensor.data_ptr, tensors))
     except TypeError:  # not torch tensors: anything with a data_ptr()
