@@ -270,11 +270,6 @@ __device__ __forceinline__ f32x2 add2_rd(f32x2 x, f32x2 y) {
   asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
   return r;
 }
-__device__ __forceinline__ f32x2 add2_ru(f32x2 x, f32x2 y) {
-  f32x2 r;
-  asm("add.rp.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
-  return r;
-}
 __device__ __forceinline__ f32x2 fma2_rn(f32x2 x, f32x2 y, f32x2 z) {
   f32x2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
@@ -1493,27 +1488,30 @@ __device__ __forceinline__ uint32_t e2m1x2_rn(float x0, float x1) {
   return p;
 }
 
-// Stochastic E2M1 code shared by every value of an interval of magnitudes
-// [xm, xM] (sign: that of q), decided from its smaller end xm alone, given
-// lim = 2^32 - W with W >= 2 (xM - xm) 2^32 + 1.  In xm's binade the grid
-// position is Q = |x| rsp (rsp = 2, 1, 1/2 on [0, 2), [2, 4), [4, 6]; 6 and
-// above saturate at Q = 3), exact in binary32; with k its integer part and
-// F = floor(frac(Q) 2^32), the code is off + k + [r < F].  Every binade edge
-// and the saturation point lie at an integer Q of xm's scale, and Q 2^32
-// grows by less than W over the interval (slope rsp <= 2); so when F + W and
-// ((F + 2^32 - 1 - r) mod 2^32) + W both stay below 2^32, no value of the
-// interval crosses a step or changes its rounding decision (same = true).
-// xm <= 0 or NaN (an interval reaching zero) reports false.
-__device__ __forceinline__ uint32_t e2m1_sr_interval(float xm, float q, uint32_t r, uint32_t lim, bool& same) {
-  const float am = fminf(xm, 6.0f);
-  const float rsp = am < 2.0f ? 2.0f : (am < 4.0f ? 1.0f : 0.5f);
-  const uint32_t off = am < 2.0f ? 0u : (am < 4.0f ? 2u : 4u);
-  const float qq = __fmul_rn(am, rsp);  // exact (a power of two)
-  const float kf = truncf(qq);
-  const uint32_t F = __float2uint_rz(__fmul_rn(__fsub_rn(qq, kf), 4294967296.0f));  // exact
-  const uint32_t sl = F + ~r;
-  same = xm > 0.0f && max(F, sl) < lim;
-  return ((__float_as_uint(q) >> 28) & 8u) | (__float2uint_rz(kf) + off + (r < F ? 1u : 0u));
+// Stochastic E2M1 code (magnitude) shared by every value of an interval of
+// magnitudes [xm, xM], decided from its smaller end xm > 0 alone.  The grid
+// position P(x), one unit a code, is read off binary32's own bits: over
+// [1, 2), [2, 4) and [4, 6] the codes are the exponent and the top mantissa bit
+// (bits 22 up, less a constant), and over [0, 1) those of 1 + x; the 22 bits
+// below are the fraction, in ticks of 2^-22.  P is continuous and rises by at
+// most 2^23 ticks per unit of x; 6 and above stay at P = 7.  A value steps up
+// iff r < floor(frac 2^32), so its code is the integer part of P plus 2^32 - 1 -
+// r in units of 2^-32; returned is s, that sum in whole ticks rounded down (1 +
+// xm is too).  With ticks >= (xM - xm) 2^23 + 3 (one tick each for the rounding
+// of 1 + xm, of P and of r), the sums of the whole interval lie in [s, s +
+// ticks + 1 tick's remainder), so the code is s >> 22 for all of it unless
+// (s ^ (s + ticks)) >> 22 is set.
+// The stochastic encode is bound by issue slots, and this form converts nothing
+// between binary32 and integers (three quarter-rate conversions an element
+// when the integer part and fraction were taken apart): a list of 0.54 B
+// weights, linear layers in NVFP4 with compute copies and binary32 moments,
+// 2455 us before, 2375 now (2345 at the copy bandwidth).
+__device__ __forceinline__ uint32_t e2m1_sr_ticks(float xm, uint32_t r) {
+  const float a = fminf(xm, 6.0f);
+  const bool sub = a < 1.0f;
+  const float z = sub ? __fadd_rd(a, 1.0f) : a;
+  // 2^22 - 1 less the bits of P = 0 on this side: 1.0f's for 1 + x, 0.5f's (two codes below 1.0f's) for x
+  return __float_as_uint(z) + (sub ? 0x003FFFFFu - 0x3F800000u : 0x003FFFFFu - 0x3F000000u) - (r >> 10);
 }
 
 // A block scale code with the two products its covering test and the encode
@@ -1713,28 +1711,39 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
       if (SR) {
         uint32_t rnd[8];
         group_random_bits<kNVFP4>(a, gi << 3, rnd);
-        // lim = 2^32 - W for the group.  An interval's magnitudes span
-        // xM - xm <= 3.5 e2: 2 e2 from ends() (e2 its bound), one directed
-        // rounding at each end (each within e2 / 8, since e2 >= |q| 2^-20)
-        // and the lower end below taken |q| 2^-20 lower still.  With e2 <=
-        // (8 2^-20 + ei)(1 + 2^-23) while |q| <= 8, 2 (xM - xm) 2^32 + 1 <=
-        // (2^-17 + ei) 2^35 + 2.  Larger |q| saturates at both ends (or, with
-        // ei > 1, leaves lim = 0: nothing is certified).
-        const uint32_t lim =
+        // The group's ticks.  An interval's magnitudes span xM - xm <= 3.5 e2:
+        // 2 e2 from ends() (e2 its bound), one directed rounding at each end
+        // (each within e2 / 8, since e2 >= |q| 2^-20) and the lower end below
+        // taken |q| 2^-20 lower still.  With e2 <= (8 2^-20 + ei)(1 + 2^-23)
+        // while |q| <= 8, (xM - xm) 2^23 + 3 <= 2^8 + ei 2^25 + 3.  Larger |q|
+        // saturates at both ends; from ei = 2^-3 on nothing is certified
+        // (2^22 ticks always reach the next code).
+        const uint32_t ticks =
             ei <= 5.9604644775390625e-08f /* 2^-24 */
-                ? 4294701056u /* 2^32 - (2^18 + 2^12): W <= 2^18 + 2^11 + 2 when ei <= 2^-24 */
-                : __float2uint_rd(__fsub_rd(4294967296.0f,
-                                            __fadd_ru(__fmaf_ru(ei, 34359738368.0f /* 2^35 */, 262144.0f /* 2^18 */),
-                                                      2.0f)));
+                ? 264u
+                : __float2uint_ru(fminf(__fmaf_ru(ei, 33554432.0f /* 2^25 */, 260.0f), 4194304.0f /* 2^22 */));
         const float inv_lo = __fmul_rd(inv, 0.999998092651367188f /* 1 - 2^-19 */);
+        // a lower bound of the smaller magnitude of ends(): |wf| inv (1 - 2^-19)
+        // (below |q| (1 - 2^-20), q = wf inv rounded) less ei, rounded down
+        auto low_end = [&](int j) { return __fmaf_rd(fabsf(wf[j]), inv_lo, -ei); };
+        uint32_t cross = 0u;
+        float xmin = INFINITY;
 #pragma unroll
         for (int j = 0; j < kGroup; ++j) {
-          // a lower bound of the smaller magnitude of ends(): |wf| inv (1 - 2^-19)
-          // (below |q| (1 - 2^-20), q = wf inv rounded) less ei, rounded down
-          const float xm = __fmaf_rd(fabsf(wf[j]), inv_lo, -ei);
-          bool same;
-          packed |= e2m1_sr_interval(xm, wf[j], rnd[j], lim, same) << (4 * j);
-          if (!same) redo |= 1u << j;
+          const float xm = low_end(j);
+          const uint32_t s = e2m1_sr_ticks(xm, rnd[j]);
+          cross |= s ^ (s + ticks);
+          xmin = fminf(xmin, xm);
+          const uint32_t sign = __float_as_uint(wf[j]) >> 31;
+          packed |= ((s >> 22) & 7u) << (4 * j) | sign << (4 * j + 3);
+        }
+        if ((cross >> 22) || !(xmin > 0.0f)) {  // rare: which elements
+#pragma unroll
+          for (int j = 0; j < kGroup; ++j) {
+            const float xm = low_end(j);
+            const uint32_t s = e2m1_sr_ticks(xm, rnd[j]);
+            if (((s ^ (s + ticks)) >> 22) || !(xm > 0.0f)) redo |= 1u << j;
+          }
         }
       } else {  // two elements at a time, both ends
         uint32_t diff = 0u;

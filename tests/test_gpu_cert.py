@@ -112,3 +112,24 @@ def test_options_in_every_format(name, rnd, hp):
     mt.ve[big][17::1009] = float("inf")
     wl = mt.workload
     _steps(P().Run(wl, mt=mt, hp=hp), 2, f"{name}/{rnd}/{hp}")
+
+
+# Stochastic E2M1 codes read off binary32's bits, where that can go wrong:
+# weights that a small step leaves beside a code (so beside zero, beside 1,
+# where 1 + x takes over from x, beside the binade edges 2 and 4 and the
+# saturation point 6), steps from far below a tick of 2^-22 to several codes
+# (an error bound ei from under 2^-24, one constant, to past 2^-3, nothing
+# certified), and enough elements that some random bits lie at the decision
+@pytest.mark.parametrize("md", ["f32", "bf16"])
+@pytest.mark.parametrize("lr", [1e-7, 1e-4, 1e-2, 1e2, 1e5])
+def test_stochastic_e2m1_codes_beside_the_grid(lr, md):
+    wl = W.Workload(name="grid", specs=tuple(W.TensorSpec(f"t{i}", n, "matrix") for i, n in enumerate((200000, 3840, 97))),
+                    weight_dtype="nvfp4", grad_dtype="bf16", moment_dtype=md, rounding="stochastic", steps=2, seed=23,
+                    zero_frac=0.0, grad=("normal_logu", 1e-6, 1e-1), compute_copy=True)
+    mt = W.materialize(wl, "cpu", warm_state=True)
+    gen = torch.Generator().manual_seed(5)
+    for k in range(len(mt.w)):
+        mt.w[k].copy_(torch.randint(0, 256, (mt.w[k].numel(),), generator=gen, dtype=torch.uint8))
+        if mt.g[k].numel() % 2:
+            mt.w[k][-1] &= 0x0F  # the spare nibble is zero
+    _steps(P().Run(wl, mt=mt, hp=dict(lr_add=lr, lr_mul=min(lr, 0.5))), 2, f"grid lr={lr}/{md}")
