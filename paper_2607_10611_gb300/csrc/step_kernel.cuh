@@ -47,30 +47,21 @@ constexpr uint32_t kSpinLimit = 1u << 22;  // mbarrier try_wait attempts before 
 // ---------------------------------------------------------------------------
 // Global memory: streaming vector stores (no L1 allocation).
 // ---------------------------------------------------------------------------
-// 256-bit stores carry the binary32 moments (nothing else uses them).  HINT
-// adds an L2 evict-first policy, chosen per kernel instance as measured (two
-// or three alternating runs each): with it the 1.5B list ran 1.4 % faster,
-// the ragged list, GPT-2 and the NVFP4 regime with RNE 0.4-0.6 %, the FP8
-// regime 0.1 % slower; the NVFP4 regime with SR (issue-bound) 1.2 % slower,
-// so its instance stores plain.  The same hint on the 128-bit stores of BF16
-// moments slowed the 7B list by 0.2 %, so those stay plain.
-template <bool HINT = true>
+// 256-bit stores carry the binary32 moments (nothing else uses them), with an
+// L2 evict-first policy, as measured (two or three alternating runs each):
+// with it the 1.5B list ran 1.4 % faster, the ragged list, GPT-2 and the NVFP4
+// regime with RNE 0.4-0.6 %, the FP8 regime 0.1 % slower, the NVFP4 regime
+// with SR (0.54 B weights) 1.2 % faster, 2375 -> 2348 us.  The same hint on the
+// 128-bit stores of BF16 moments slowed the 7B list by 0.2 %, so those stay
+// plain.
 __device__ __forceinline__ void st8(void* p, const uint32_t (&r)[8]) {
-  if constexpr (HINT) {
-    uint64_t pol;
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    asm volatile("st.global.L1::no_allocate.L2::cache_hint.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;"
-                 :
-                 : "l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
-                   "r"(r[6]), "r"(r[7]), "l"(pol)
-                 : "memory");
-  } else {
-    asm volatile("st.global.L1::no_allocate.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 :
-                 : "l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
-                   "r"(r[6]), "r"(r[7])
-                 : "memory");
-  }
+  uint64_t pol;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  asm volatile("st.global.L1::no_allocate.L2::cache_hint.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;"
+               :
+               : "l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
+                 "r"(r[6]), "r"(r[7]), "l"(pol)
+               : "memory");
 }
 __device__ __forceinline__ void st4(void* p, const uint32_t (&r)[4]) {
   asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};"
@@ -740,13 +731,12 @@ __device__ __forceinline__ void put_bf16(const uint32_t (&o)[4], void* g, int64_
             static_cast<uint16_t>((j & 1) ? (o[j >> 1] >> 16) : (o[j >> 1] & 0xFFFFu));
   }
 }
-template <bool HINT = true>
 __device__ __forceinline__ void put_f32(const float (&x)[8], void* g, int64_t e0, int valid, bool vec) {
   if (vec && valid == kGroup) {
     uint32_t o[8];
 #pragma unroll
     for (int j = 0; j < kGroup; ++j) o[j] = __float_as_uint(x[j]);
-    st8<HINT>(static_cast<float*>(g) + e0, o);
+    st8(static_cast<float*>(g) + e0, o);
   } else {
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
@@ -975,13 +965,13 @@ __device__ __forceinline__ void put_compute(const uint32_t (&codes)[2], float sc
 }
 
 // Store the updated moments (BF16 moments nearest-even).
-template <int MD, bool HINT = true>  // HINT: see st8
+template <int MD>
 __device__ __forceinline__ void put_moments(const TensorCtx& x, int64_t e0, int valid, const float (&m)[8],
                                             const float (&v)[8], const float (&ve)[8]) {
   if (MD == kF32) {
-    put_f32<HINT>(m, x.d.m, e0, valid, x.vec);
-    put_f32<HINT>(v, x.d.v, e0, valid, x.vec);
-    put_f32<HINT>(ve, x.d.ve, e0, valid, x.vec);
+    put_f32(m, x.d.m, e0, valid, x.vec);
+    put_f32(v, x.d.v, e0, valid, x.vec);
+    put_f32(ve, x.d.ve, e0, valid, x.vec);
   } else {
     uint32_t om[4], ov[4], oe[4];
 #pragma unroll
@@ -1505,7 +1495,7 @@ __device__ __forceinline__ uint32_t e2m1x2_rn(float x0, float x1) {
 // between binary32 and integers (three quarter-rate conversions an element
 // when the integer part and fraction were taken apart): a list of 0.54 B
 // weights, linear layers in NVFP4 with compute copies and binary32 moments,
-// 2455 us before, 2375 now (2345 at the copy bandwidth).
+// 2455 us before, 2375 after (2345 at the copy bandwidth).
 __device__ __forceinline__ uint32_t e2m1_sr_ticks(float xm, uint32_t r) {
   const float a = fminf(xm, 6.0f);
   const bool sub = a < 1.0f;
@@ -1666,7 +1656,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
         if ((vmask >> (2 * i + 1)) & 1u) am = fmaxf(am, fabsf(wf[2 * i + 1]));
       }
     }
-    if constexpr (SRC != kExactRegs) put_moments<MD, !SR>(x, e0, valid, m, v, ve);
+    if constexpr (SRC != kExactRegs) put_moments<MD>(x, e0, valid, m, v, ve);
     const float et = -nt;
     const uint32_t bad = cert_not_finite(fin) ? vmask : 0u;
     const float lo_t = bad ? 0.0f : fmaxf(__fsub_rd(am, et), 0.0f);
@@ -1775,7 +1765,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
         }
       }
     }
-    if constexpr (SRC == kExactRegs) put_moments<MD, !SR>(x, e0, valid, m, v, ve);
+    if constexpr (SRC == kExactRegs) put_moments<MD>(x, e0, valid, m, v, ve);
   } else {
     float wn[8];
     uint32_t amx = 0u;
@@ -1794,7 +1784,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
       packed |= (e2m1_encode<SR>(__fdiv_rn(wn[j], d), SR ? rnd[j] : 0u) & 0xFu) << (4 * j);
-    put_moments<MD, !SR>(x, e0, valid, m, v, ve);
+    put_moments<MD>(x, e0, valid, m, v, ve);
   }
   put_fp4(packed, x.d.w, e0, valid, x.vec);
   if ((threadIdx.x & 1) == 0 && valid > 0) static_cast<uint8_t*>(x.scale)[e0 / kFp4Block] = static_cast<uint8_t>(c_new);
