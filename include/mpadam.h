@@ -296,6 +296,16 @@ int32_t mpadam_debug_tile_schedule(const int64_t* numel, int32_t n, int32_t ctas
                                    int32_t chunk_tiles, int64_t* cta_runs, int32_t* cta_first,
                                    int64_t* pool, int32_t pool_cap, int32_t* pool_count);
 
+/* Host only, no GPU: the shared-memory ring of the step kernel for cfg's
+ * formats (weight_dtype may be any of the four) in a block of smem_bytes
+ * bytes; misaligned != 0: of the instance for misaligned gradients or
+ * one-byte weights (NVFP4 has none).  layout receives 8 values: stages, bytes
+ * of one stage, the offsets inside a stage of the gradients, mu, nu, nu_e and
+ * the block scales (the weights start at 0), and the static shared memory
+ * beside the ring.  Errors: EINVAL, EUNSUPPORTED (fewer than two stages). */
+int32_t mpadam_debug_ring_layout(const mpadam_config* cfg, int32_t misaligned, int32_t smem_bytes,
+                                 int32_t* layout);
+
 /* Frees the library's metadata (synchronises the device first).  NULL is a
  * no-op.  Never touches caller-owned tensors. */
 int32_t mpadam_destroy(mpadam_state* s);

@@ -26,7 +26,8 @@ EXPORTED = ["mpadam_create", "mpadam_create_ex", "mpadam_fp8_init", "mpadam_step
             "mpadam_destroy", "mpadam_last_error", "mpadam_global_offset", "mpadam_global_length", "mpadam_set_grid",
             "mpadam_set_tail_pool", "mpadam_launch_info", "mpadam_rng_lanes", "mpadam_step_noalloc", "mpadam_noalloc_status", "mpadam_device_status",
             "mpadam_toy_create", "mpadam_toy_step", "mpadam_toy_run", "mpadam_toy_status", "mpadam_toy_destroy",
-            "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation", "mpadam_debug_tile_schedule"]
+            "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation",
+            "mpadam_debug_tile_schedule", "mpadam_debug_ring_layout"]
 
 
 class MPAdamError(RuntimeError):
@@ -127,6 +128,7 @@ def lib() -> ctypes.CDLL:
             "mpadam_host_buffer_free": [P, i64],
             "mpadam_debug_fail_allocation": [i32],
             "mpadam_debug_tile_schedule": [P, i32, i32, i32, i32, P, P, P, i32, P],
+            "mpadam_debug_ring_layout": [P, i32, i32, P],
         }
         for name, args in sig.items():
             f = getattr(L, name)
@@ -336,3 +338,10 @@ def mpadam_debug_tile_schedule(numel, ctas: int, static_q: int, chunk_tiles: int
             continue
         _check(rc)
         return runs, first, pool[:count.value]
+
+
+def mpadam_debug_ring_layout(cfg: mpadam_config, misaligned: bool, smem_bytes: int) -> dict:
+    """The step kernel's shared-memory ring, computed on the host."""
+    out = (ctypes.c_int32 * 8)()
+    _check(lib().mpadam_debug_ring_layout(ctypes.byref(cfg), int(misaligned), smem_bytes, out))
+    return dict(zip(("stages", "stage_bytes", "off_g", "off_m", "off_v", "off_ve", "off_s", "static_bytes"), out))

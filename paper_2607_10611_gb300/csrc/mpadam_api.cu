@@ -153,14 +153,12 @@ void round_keys(uint64_t seed, uint32_t* rk0, uint32_t* rk1) {
   }
 }
 
-// Shared-memory ring of the step kernel: one stage holds one tile of every
-// array (w | g | mu | nu | nu_e | block scales); as many stages as fit, 2 to
-// kMaxStages.
+// Shared-memory ring of a step kernel instance: one stage holds one tile of
+// every array (w | g | mu | nu | nu_e | block scales); as many stages as fit,
+// 2 to kMaxStages.
 struct Geometry {
   int32_t stages = 0, stage_bytes = 0, off_g = 0, off_m = 0, off_v = 0, off_ve = 0, off_s = 0, dyn_smem = 0;
 };
-
-int32_t make_geometry(const mpadam_config& c, int32_t wd, int dev, Geometry* g);
 
 bool kernel_options(const mpadam_config& c) {
   return std::isfinite(c.g_max) || std::isfinite(c.w_max) || c.wd_add != 0.0f;
@@ -200,28 +198,37 @@ int32_t check_config(const mpadam_config* c, bool per_tensor_weights = false) {
   return MPADAM_OK;
 }
 
-int32_t make_geometry(const mpadam_config& c, int32_t wd, int dev, Geometry* g) {
+// The ring of the instance for (or not for) misaligned arrays, in a block of at
+// most `smem` bytes of shared memory.  Misaligned one-byte weights and
+// gradients keep their place modulo 16 bytes, so those regions take a line
+// more, and only there: with it, a fourth stage of block-scaled E4M3 with BF16
+// gradients and binary32 moments would miss the block's limit by 64 bytes
+// (GB300: 232,448).
+int32_t ring_layout(const mpadam_config& c, int32_t wd, bool mis, int32_t smem, Geometry* g) {
   const int32_t rw = (int32_t)weight_bytes(wd, mpadam::kTile);
   const int32_t rg = mpadam::kTile * (int32_t)elem_size(c.grad_dtype);
   const int32_t rm = mpadam::kTile * (int32_t)elem_size(c.moment_dtype);
   const int32_t rs = wd == MPADAM_E4M3_B32 ? mpadam::kTileBlocks * 2           // 240 bytes, a 16-byte multiple
                    : wd == MPADAM_NVFP4    ? mpadam::kTileFp4Blocks               // 240 bytes
                                            : 0;
-  // one-byte weights and gradients keep their place modulo 16 bytes: up to a line more
-  g->off_g = rw + (wd == MPADAM_E4M3 || wd == MPADAM_E4M3_B32 ? 16 : 0);
-  g->off_m = g->off_g + rg + 16;
+  const int32_t line = mis ? 16 : 0;
+  g->off_g = rw + (wd == MPADAM_E4M3 || wd == MPADAM_E4M3_B32 ? line : 0);
+  g->off_m = g->off_g + rg + line;
   g->off_v = g->off_m + rm;
   g->off_ve = g->off_v + rm;
   g->off_s = g->off_ve + rm;
   g->stage_bytes = g->off_s + rs;
-  int optin = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute(MaxSharedMemoryPerBlockOptin)");
-  const int32_t budget = optin - 1024;  // static barriers (128 bytes) and slack
-  g->stages = std::min<int32_t>(mpadam::kMaxStages, budget / g->stage_bytes);
+  g->stages = std::min<int32_t>(mpadam::kMaxStages, (smem - mpadam::kStaticSmem) / g->stage_bytes);
   if (g->stages < 2) return fail(MPADAM_EUNSUPPORTED, "device shared memory too small for the step pipeline");
   g->dyn_smem = g->stages * g->stage_bytes;
   return MPADAM_OK;
+}
+
+int32_t make_geometry(const mpadam_config& c, int32_t wd, bool mis, int dev, Geometry* g) {
+  int optin = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute(MaxSharedMemoryPerBlockOptin)");
+  return ring_layout(c, wd, mis, optin, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -317,7 +324,7 @@ struct Group {
   const void* kernel = nullptr;
   const void* kernel_mis = nullptr;     // the instance for misaligned gradients or one-byte weights
   bool w_mis = false;                   // one-byte weights among them that are not 16-byte aligned
-  Geometry geo;
+  Geometry geo, geo_mis;
   int32_t default_grid = 0, grid = 0;
   int32_t* d_cta_first = nullptr;
   int32_t cta_cap = 0;
@@ -572,9 +579,9 @@ void fill_step(StepArgs& a, const mpadam_config& cfg, int64_t step) {
   a.a_zero_slot = (int32_t)((step + 2) % 3);
 }
 
-StepArgs base_args(const mpadam_state* s, const Group& g) {
+StepArgs base_args(const mpadam_state* s, const Group& g, bool mis) {
   StepArgs a;
-  fill_common(a, s->cfg, g.geo, g.tiles, s->n, s->fp8_exp, s->fp8_amax);
+  fill_common(a, s->cfg, mis ? g.geo_mis : g.geo, g.tiles, s->n, s->fp8_exp, s->fp8_amax);
   a.desc = s->d_desc + g.first;
   a.n_desc = g.count;
   a.aux = g.aux ? s->d_aux + g.first : nullptr;
@@ -728,9 +735,10 @@ int32_t create_state(const std::vector<TensorIn>& t, const mpadam_config* cfg, i
       for (const TensorDesc& d : g.h_desc)
         g.w_mis = g.w_mis || ((g.wd == MPADAM_E4M3 || g.wd == MPADAM_E4M3_B32) && d.numel > 0 && !is_aligned(d.w, 16));
       if (!g.kernel || !g.kernel_mis) { release(s); return fail(MPADAM_EUNSUPPORTED, "no kernel for these formats"); }
-      rc = make_geometry(*cfg, g.wd, s->device, &g.geo);
+      rc = make_geometry(*cfg, g.wd, false, s->device, &g.geo);
+      if (!rc) rc = make_geometry(*cfg, g.wd, g.kernel_mis != g.kernel, s->device, &g.geo_mis);
       if (rc) { release(s); return rc; }
-      rc = prepare_kernel(g.kernel_mis, g.geo, s->sm_count, &g.default_grid);
+      rc = prepare_kernel(g.kernel_mis, g.geo_mis, s->sm_count, &g.default_grid);
       if (!rc) rc = prepare_kernel(g.kernel, g.geo, s->sm_count, &g.default_grid);
       if (rc) { release(s); return rc; }
     }
@@ -817,7 +825,10 @@ cudaError_t launch_kernel(const void* kernel, int32_t grid, void** params, int32
 // One launch of a group's step kernel over its tiles [tile_base, tile_base + count).
 int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t stream, int64_t tile_base,
                     int64_t count, const int32_t* cta_first, int32_t grid, uint32_t* pool_next = nullptr) {
-  StepArgs a = base_args(s, g);
+  bool mis = g.w_mis;
+  for (int32_t p = g.first; !mis && p < g.first + g.count; ++p)
+    mis = s->numel[s->order[p]] > 0 && !is_aligned(s->h_grads[p], 16);
+  StepArgs a = base_args(s, g, mis);
   a.cta_first = cta_first;
   a.tile_base = tile_base;
   a.total_tiles = count;
@@ -840,10 +851,8 @@ int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t 
   }
   fill_step(a, s->cfg, step);
   void* params[] = {&a};
-  bool mis = g.w_mis;
-  for (int32_t p = g.first; !mis && p < g.first + g.count; ++p)
-    mis = s->numel[s->order[p]] > 0 && !is_aligned(s->h_grads[p], 16);
-  cudaError_t e = launch_kernel(mis ? g.kernel_mis : g.kernel, grid, params, g.geo.dyn_smem, stream);
+  cudaError_t e = launch_kernel(mis ? g.kernel_mis : g.kernel, grid, params,
+                                mis ? g.geo_mis.dyn_smem : g.geo.dyn_smem, stream);
   if (e != cudaSuccess) return cuda_fail(e, "launch of the step kernel");
   return MPADAM_OK;
 }
@@ -1070,7 +1079,7 @@ int32_t mpadam_fp8_init(mpadam_state* s, const int32_t* init_exp, int64_t first_
   e = cudaMemsetAsync(s->fp8_amax, 0, sizeof(uint32_t) * 3 * (size_t)s->n, stream);
   if (e != cudaSuccess) return cuda_fail(e, "clearing fp8_amax");
   if (g->tiles == 0) return MPADAM_OK;
-  StepArgs a = base_args(s, *g);
+  StepArgs a = base_args(s, *g, false);
   int32_t exp_slot = (int32_t)(first_step % 2), amax_slot = (int32_t)(first_step % 3);
   void* params[] = {&a, &exp_slot, &amax_slot};
   e = cudaLaunchKernel(reinterpret_cast<const void*>(&fp8_amax_kernel), dim3(g->grid), dim3(mpadam::kConsumers),
@@ -1345,7 +1354,7 @@ extern "C" int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, 
   const void* kernel = select_kernel(*cfg, cfg->weight_dtype, mis);
   if (!kernel) return fail(MPADAM_EUNSUPPORTED, "no kernel for these formats");
   Geometry geo;
-  rc = make_geometry(*cfg, cfg->weight_dtype, dev, &geo);
+  rc = make_geometry(*cfg, cfg->weight_dtype, mis, dev, &geo);
   if (rc) return rc;
   int32_t grid = 0;
   rc = prepare_kernel(kernel, geo, sms, &grid);
@@ -1622,6 +1631,21 @@ extern "C" int32_t mpadam_host_buffer_free(void* ptr, int64_t bytes) {
 extern "C" int32_t mpadam_debug_fail_allocation(int32_t after) {
   if (after < -1) return fail(MPADAM_EINVAL, "after must be >= -1");
   g_fail_countdown.store(after);
+  return MPADAM_OK;
+}
+
+extern "C" int32_t mpadam_debug_ring_layout(const mpadam_config* cfg, int32_t misaligned, int32_t smem_bytes,
+                                            int32_t* layout) {
+  int32_t rc = check_config(cfg, true);
+  if (rc) return rc;
+  if (cfg->weight_dtype < MPADAM_BF16 || cfg->weight_dtype > MPADAM_NVFP4)
+    return fail(MPADAM_EINVAL, "weight_dtype must be MPADAM_BF16, MPADAM_E4M3, MPADAM_E4M3_B32 or MPADAM_NVFP4");
+  if (!layout || smem_bytes < 0) return fail(MPADAM_EINVAL, "layout is NULL or smem_bytes < 0");
+  Geometry g;
+  rc = ring_layout(*cfg, cfg->weight_dtype, misaligned != 0, smem_bytes, &g);
+  if (rc) return rc;
+  const int32_t out[8] = {g.stages, g.stage_bytes, g.off_g, g.off_m, g.off_v, g.off_ve, g.off_s, mpadam::kStaticSmem};
+  std::memcpy(layout, out, sizeof out);
   return MPADAM_OK;
 }
 

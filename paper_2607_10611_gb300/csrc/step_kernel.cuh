@@ -809,7 +809,9 @@ struct StageHead {
   uint32_t seed;
   uint32_t w_range, g_range;  // what was copied of the weights (not kNVFP4) and gradients (staged_range)
 };
-static_assert(sizeof(StageHead) * kMaxStages + 16 * kMaxStages <= 1024, "static shared memory (make_geometry leaves 1 KB)");
+// What the kernel holds beside the ring: the heads and two barriers per stage.
+constexpr int kStaticSmem = kMaxStages * (static_cast<int>(sizeof(StageHead)) + 16);
+static_assert(kStaticSmem == 1024, "no padding between them");
 
 // Per-tensor values the consumers keep while walking a tensor's tiles.
 struct TensorCtx {
