@@ -719,16 +719,26 @@ __device__ __forceinline__ void get_e4m3(float (&x)[8], uint32_t saddr, float sc
   for (int j = 0; j < kGroup; ++j) x[j] = __fmul_rn(x[j], scale);
 }
 
-// Group stores (vector when whole and aligned, else element by element).
+// Group stores (vector when whole and aligned, else element by element).  The
+// single stores are volatile so that those of one array stay together and L1
+// merges them by sector (217 M parameters, BF16 moments, BF16 weights 2 bytes
+// off a line: 1647 -> 1507 us).
+__device__ __forceinline__ void st_u32(void* p, uint32_t v) {
+  asm volatile("st.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_u16(void* p, uint32_t v) {
+  asm volatile("{\n .reg .b16 h;\n cvt.u16.u32 h, %1;\n st.global.u16 [%0], h;\n}" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_u8(void* p, uint32_t v) {
+  asm volatile("st.global.u8 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void put_bf16(const uint32_t (&o)[4], void* g, int64_t e0, int valid, bool vec) {
   if (vec && valid == kGroup) {
     st4(static_cast<uint16_t*>(g) + e0, o);
   } else {
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
-      if (j < valid)
-        static_cast<uint16_t*>(g)[e0 + j] =
-            static_cast<uint16_t>((j & 1) ? (o[j >> 1] >> 16) : (o[j >> 1] & 0xFFFFu));
+      if (j < valid) st_u16(static_cast<uint16_t*>(g) + e0 + j, (j & 1) ? (o[j >> 1] >> 16) : (o[j >> 1] & 0xFFFFu));
   }
 }
 __device__ __forceinline__ void put_f32(const float (&x)[8], void* g, int64_t e0, int valid, bool vec) {
@@ -740,7 +750,7 @@ __device__ __forceinline__ void put_f32(const float (&x)[8], void* g, int64_t e0
   } else {
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
-      if (j < valid) static_cast<float*>(g)[e0 + j] = x[j];
+      if (j < valid) st_u32(static_cast<float*>(g) + e0 + j, __float_as_uint(x[j]));
   }
 }
 __device__ __forceinline__ void put_e4m3(const uint32_t (&o)[2], void* g, int64_t e0, int valid, bool vec) {
@@ -749,7 +759,7 @@ __device__ __forceinline__ void put_e4m3(const uint32_t (&o)[2], void* g, int64_
   } else {
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
-      if (j < valid) static_cast<uint8_t*>(g)[e0 + j] = static_cast<uint8_t>(o[j >> 2] >> (8 * (j & 3)));
+      if (j < valid) st_u8(static_cast<uint8_t*>(g) + e0 + j, o[j >> 2] >> (8 * (j & 3)));
   }
 }
 
@@ -813,12 +823,20 @@ struct StageHead {
 constexpr int kStaticSmem = kMaxStages * (static_cast<int>(sizeof(StageHead)) + 16);
 static_assert(kStaticSmem == 1024, "no padding between them");
 
+// The arrays that a step writes.  Each is stored by vectors when it is aligned
+// itself, as each is read from the stage when it is there (load_group), so one
+// array off its boundary costs its own accesses alone: 217 M parameters, BF16
+// weights and gradients, binary32 moments (aligned 1152 us) with the weights 2
+// bytes off a line 2644 -> 1204 us, with mu 8 bytes off 2640 -> 1217; with
+// BF16 moments 2479 -> 1507 and 2598 -> 1506.
+constexpr uint32_t kVecW = 1, kVecM = 2, kVecV = 4, kVecVe = 8, kVecCc = 16, kVecAll = 31;
+
 // Per-tensor values the consumers keep while walking a tensor's tiles.
 struct TensorCtx {
   TensorDesc d;        // w, m, v, ve, goff, ring
   const void* g;       // kNVFP4's exact branch (the others read gradients from the stage, or through its head)
   uint32_t gsh, wsh;   // MIS: misalign() of the gradients and of one-byte weights
-  bool vec;            // every array that is written is aligned for vector stores of whole groups
+  uint32_t vec;        // kVec* of the written arrays that are aligned for vector stores of whole groups
   bool fast;           // whole warps of a tile are staged, and stored with vector stores
   float dec_scale, enc_scale;
   float cc_scale;      // E4M3 per-tensor: 2^e of the new encode (compute copy)
@@ -839,9 +857,12 @@ __device__ __forceinline__ void load_tensor(const StageHead& h, TensorCtx& c) {
   c.g = h.g;
   c.gsh = MIS ? misalign(h.g) : 0u;
   c.wsh = MIS && (WD == kE4M3 || WD == kE4M3B) ? misalign(h.w) : 0u;
-  c.vec = aligned(c.d.w, WD == kBF16 ? 16 : (WD == kNVFP4 ? 4 : 8)) && aligned(c.d.m, MD == kF32 ? 32 : 16) &&
-          aligned(c.d.v, MD == kF32 ? 32 : 16) && aligned(c.d.ve, MD == kF32 ? 32 : 16);
-  c.fast = c.vec && (MIS || (aligned(c.d.w, 16) && aligned(c.g, 16)));
+  c.vec = kVecAll;
+  if (!aligned(c.d.w, WD == kBF16 ? 16 : (WD == kNVFP4 ? 4 : 8))) c.vec &= ~kVecW;
+  if (!aligned(c.d.m, MD == kF32 ? 32 : 16)) c.vec &= ~kVecM;
+  if (!aligned(c.d.v, MD == kF32 ? 32 : 16)) c.vec &= ~kVecV;
+  if (!aligned(c.d.ve, MD == kF32 ? 32 : 16)) c.vec &= ~kVecVe;
+  c.fast = c.vec == kVecAll && (MIS || (aligned(c.d.w, 16) && aligned(c.g, 16)));
   c.dec_scale = c.enc_scale = c.cc_scale = 1.0f;
   c.scale = nullptr;
   c.cc = nullptr;
@@ -853,7 +874,7 @@ __device__ __forceinline__ void load_tensor(const StageHead& h, TensorCtx& c) {
     c.gscale = h.gscale;
     // the compute copy joins the vector path only when 16-byte aligned;
     // block scales are staged (whole tiles: 240 bytes) only when 16-byte aligned
-    if (c.cc && !aligned(c.cc, 16)) c.vec = c.fast = false;
+    if (c.cc && !aligned(c.cc, 16)) { c.vec &= ~kVecCc; c.fast = false; }
     if ((WD == kE4M3B || WD == kNVFP4) && !aligned(c.scale, 16)) c.fast = false;
   }
 }
@@ -887,66 +908,96 @@ __device__ __forceinline__ void patch_group(const StepArgs& a, const TensorCtx& 
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// One array's eight elements of a group, each in a word of its own (a BF16 or a
+// code in the low bits): from the stage when the group's bytes are there, else
+// from global memory (elements from `valid` on are 0).
+template <int ES, bool SHIFT>
+__device__ __forceinline__ void raw_group(uint32_t (&r)[8], bool staged, uint32_t saddr, const void* p, int64_t e0,
+                                          int valid) {
+  if (staged) {
+    if (SHIFT) {
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j)
+        r[j] = ES == 4 ? lds_u32(saddr + 4u * j) : (ES == 2 ? lds_u16(saddr + 2u * j) : lds_u8(saddr + j));
+    } else if (ES == 4) {
+      uint32_t a[4], b[4];
+      lds4(saddr, a);
+      lds4(saddr + 16, b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { r[i] = a[i]; r[4 + i] = b[i]; }
+    } else if (ES == 2) {
+      uint32_t t[4];
+      lds4(saddr, t);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { r[2 * i] = t[i] & 0xFFFFu; r[2 * i + 1] = t[i] >> 16; }
+    } else {
+      uint32_t t[2];
+      lds2(saddr, t);
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) r[j] = (t[j >> 2] >> (8 * (j & 3))) & 0xFFu;
+    }
+    return;
+  }
+  const uint8_t* q = static_cast<const uint8_t*>(p) + e0 * ES;
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    if (ES == 4) r[j] = j < valid ? *reinterpret_cast<const uint32_t*>(q + 4 * j) : 0u;
+    else if (ES == 2) r[j] = j < valid ? *reinterpret_cast<const uint16_t*>(q + 2 * j) : 0u;
+    else r[j] = j < valid ? q[j] : 0u;
+  }
+}
+
 // One group of a partial tile, or of a tensor whose arrays are not all staged
-// or aligned: every array from the stage when all of them hold the whole group
-// there, else all of them element by element from global memory -- the loads
-// of all arrays before the first use, so that the group waits on memory once
-// (array by array it waited five times: a BF16-moment list of 4000 ragged
-// tensors took 345 us, now 295).  dec: the scale the codes decode with.
+// or aligned: each array from the stage when it holds the whole group there,
+// else element by element from global memory -- the loads of all arrays before
+// the first use, so that the group waits on memory once (waiting array by
+// array, a BF16-moment list of 4000 ragged tensors took 345 us, now 295), and
+// one array's after another's, as L1, a few KB a warp beside the ring, holds
+// few arrays' lines at a time.  8-byte loads where the alignment allows them
+// were slower (binary32 moments, mu 8 bytes off: 2219 us against 1986, either
+// with all stores single).  dec: the scale the codes decode with.
 template <int WD, int GD, int MD, bool MIS>
 __device__ __forceinline__ void load_group(const StepArgs& a, const TensorCtx& x, const StageHead& h, int64_t e0,
                                            int count, int c, int valid, uint32_t st, float dec, float (&w)[8],
                                            float (&g)[8], float (&m)[8], float (&v)[8], float (&ve)[8]) {
-  constexpr int GS = esize_of(GD), MS = esize_of(MD);
+  constexpr int WS = esize_of(WD), GS = esize_of(GD), MS = esize_of(MD);
   const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
-  const uint32_t wo = WD == kNVFP4 ? 4u * c : static_cast<uint32_t>(kGroup * esize_of(WD)) * c + x.wsh;
-  const uint32_t go = kGroup * GS * c + x.gsh;
-  bool in;
-  if (MIS) in = in_range(h.w_range, wo, kGroup * esize_of(WD)) && (wo & (WD == kBF16 ? 15u : 7u)) == 0u &&
-                in_range(h.g_range, go, kGroup * GS);
-  else in = (WD == kNVFP4 ? end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1)
-                          : end * esize_of(WD) <= staged_bytes(x.d.w, count, esize_of(WD))) &&
-            end * GS <= staged_bytes(h.g, count, GS);
-  if (in && end * MS <= staged_bytes(x.d.m, count, MS) && end * MS <= staged_bytes(x.d.v, count, MS) &&
-      end * MS <= staged_bytes(x.d.ve, count, MS)) {
-    if (WD == kBF16) get_bf16(w, st + wo);
-    else if (WD == kNVFP4) get_fp4(w, st + wo, dec);
-    else get_e4m3(w, st + wo, dec);
-    if (MIS && GD == kF32) get_f32_at(g, st + a.off_g + go);
-    else if (MIS) get_bf16_at(g, st + a.off_g + go);
-    else if (GD == kF32) get_f32(g, st + a.off_g + go);
-    else get_bf16(g, st + a.off_g + go);
-    if (MD == kF32) {
-      get_f32(m, st + a.off_m + kGroup * MS * c);
-      get_f32(v, st + a.off_v + kGroup * MS * c);
-      get_f32(ve, st + a.off_ve + kGroup * MS * c);
-    } else {
-      get_bf16(m, st + a.off_m + kGroup * MS * c);
-      get_bf16(v, st + a.off_v + kGroup * MS * c);
-      get_bf16(ve, st + a.off_ve + kGroup * MS * c);
-    }
-    return;
-  }
-  auto raw = [&](const void* p, int es, int64_t i) -> uint32_t {
-    return es == 4 ? static_cast<const uint32_t*>(p)[i]
-                   : (es == 2 ? static_cast<const uint16_t*>(p)[i] : static_cast<const uint8_t*>(p)[i]);
-  };
+  const uint32_t go = kGroup * GS * c + x.gsh, mo = kGroup * MS * c;
+  const bool g_in = MIS ? in_range(h.g_range, go, kGroup * GS) : end * GS <= staged_bytes(h.g, count, GS);
   uint32_t rw[8], rg[8], rm[8], rv[8], re[8];
+  if (WD == kNVFP4) {  // the group's codes as the bytes of one word
+    rw[0] = 0u;
+    if (end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1)) {
+      rw[0] = lds_u32(st + 4u * c);
+    } else {
+      const uint8_t* q = static_cast<const uint8_t*>(x.d.w) + (e0 >> 1);
 #pragma unroll
-  for (int j = 0; j < kGroup; ++j) {
-    const bool in = j < valid;
-    rw[j] = in ? raw(x.d.w, WD == kBF16 ? 2 : 1, WD == kNVFP4 ? (e0 + j) >> 1 : e0 + j) : 0u;
-    rg[j] = in ? raw(h.g, GS, e0 + j) : 0u;
-    rm[j] = in ? raw(x.d.m, MS, e0 + j) : 0u;
-    rv[j] = in ? raw(x.d.v, MS, e0 + j) : 0u;
-    re[j] = in ? raw(x.d.ve, MS, e0 + j) : 0u;
+      for (int i = 0; i < 4; ++i) rw[1 + i] = 2 * i < valid ? q[i] : 0u;
+      rw[0] = rw[1] | rw[2] << 8 | rw[3] << 16 | rw[4] << 24;
+    }
+  } else {
+    const uint32_t wo = static_cast<uint32_t>(kGroup * WS) * c + x.wsh;
+    const bool w_in = MIS && WD != kBF16 ? in_range(h.w_range, wo, kGroup) : end * WS <= staged_bytes(x.d.w, count, WS);
+    raw_group<WS, MIS && WD != kBF16>(rw, w_in, st + wo, x.d.w, e0, valid);
   }
+  raw_group<GS, MIS>(rg, g_in, st + a.off_g + go, h.g, e0, valid);
+  raw_group<MS, false>(rm, end * MS <= staged_bytes(x.d.m, count, MS), st + a.off_m + mo, x.d.m, e0, valid);
+  raw_group<MS, false>(rv, end * MS <= staged_bytes(x.d.v, count, MS), st + a.off_v + mo, x.d.v, e0, valid);
+  raw_group<MS, false>(re, end * MS <= staged_bytes(x.d.ve, count, MS), st + a.off_ve + mo, x.d.ve, e0, valid);
   auto val = [](uint32_t r, int es) { return __uint_as_float(es == 4 ? r : r << 16); };
+  if (WD == kNVFP4) {
+    e2m1x8_to_f32(rw[0], w);
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) w[j] = j < valid ? __fmul_rn(w[j], dec) : 0.0f;
+  } else if (WD != kBF16) {
+    const uint32_t t[2] = {rw[0] | rw[1] << 8 | rw[2] << 16 | rw[3] << 24, rw[4] | rw[5] << 8 | rw[6] << 16 | rw[7] << 24};
+    e4m3x8_to_f32(t, w);
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) w[j] = __fmul_rn(w[j], dec);
+  }
 #pragma unroll
   for (int j = 0; j < kGroup; ++j) {
     if (WD == kBF16) w[j] = val(rw[j], 2);
-    else if (WD == kNVFP4) w[j] = j < valid ? __fmul_rn(e2m1_value(((e0 + j) & 1) ? (rw[j] >> 4) : (rw[j] & 0xFu)), dec) : 0.0f;
-    else w[j] = j < valid ? __fmul_rn(e4m3_value(rw[j]), dec) : 0.0f;
     g[j] = val(rg[j], GS);
     m[j] = val(rm[j], MS);
     v[j] = val(rv[j], MS);
@@ -966,14 +1017,17 @@ __device__ __forceinline__ void put_compute(const uint32_t (&codes)[2], float sc
   put_bf16(o, cc, e0, valid, vec);
 }
 
-// Store the updated moments (BF16 moments nearest-even).
-template <int MD>
+// Store the updated moments (BF16 moments nearest-even).  FAST: a whole staged
+// warp (TensorCtx::fast), where every array is aligned: its straight-line code
+// then holds neither the tests nor the single stores (217 M parameters with
+// BF16 moments, stochastic: NVFP4 982 -> 953 us, block-scaled E4M3 909 -> 893).
+template <int MD, bool FAST>
 __device__ __forceinline__ void put_moments(const TensorCtx& x, int64_t e0, int valid, const float (&m)[8],
                                             const float (&v)[8], const float (&ve)[8]) {
   if (MD == kF32) {
-    put_f32(m, x.d.m, e0, valid, x.vec);
-    put_f32(v, x.d.v, e0, valid, x.vec);
-    put_f32(ve, x.d.ve, e0, valid, x.vec);
+    put_f32(m, x.d.m, e0, valid, FAST || (x.vec & kVecM) != 0u);
+    put_f32(v, x.d.v, e0, valid, FAST || (x.vec & kVecV) != 0u);
+    put_f32(ve, x.d.ve, e0, valid, FAST || (x.vec & kVecVe) != 0u);
   } else {
     uint32_t om[4], ov[4], oe[4];
 #pragma unroll
@@ -982,9 +1036,9 @@ __device__ __forceinline__ void put_moments(const TensorCtx& x, int64_t e0, int 
       ov[i] = bf16x2_rn(v[2 * i], v[2 * i + 1]);
       oe[i] = bf16x2_rn(ve[2 * i], ve[2 * i + 1]);
     }
-    put_bf16(om, x.d.m, e0, valid, x.vec);
-    put_bf16(ov, x.d.v, e0, valid, x.vec);
-    put_bf16(oe, x.d.ve, e0, valid, x.vec);
+    put_bf16(om, x.d.m, e0, valid, FAST || (x.vec & kVecM) != 0u);
+    put_bf16(ov, x.d.v, e0, valid, FAST || (x.vec & kVecV) != 0u);
+    put_bf16(oe, x.d.ve, e0, valid, FAST || (x.vec & kVecVe) != 0u);
   }
 }
 
@@ -1119,7 +1173,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         }
       }
     }
-    put_bf16(ow, x.d.w, e0, valid, x.vec);
+    put_bf16(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
   } else if (WD == kE4M3 && a.s.cert_ok) {
     // Certified fast path for E4M3: both ends of the bound are scaled by 2^-e
     // with outward rounding and encoded; the largest |w'| must be exact, so an
@@ -1203,8 +1257,8 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         }
       }
     }
-    put_e4m3(ow, x.d.w, e0, valid, x.vec);
-    if (x.cc) put_compute(ow, x.cc_scale, x.cc, e0, valid, x.vec);
+    put_e4m3(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
+    if (x.cc) put_compute(ow, x.cc_scale, x.cc, e0, valid, STAGED || (x.vec & kVecCc) != 0u);
   } else {
   float wn[8];
 #pragma unroll
@@ -1220,7 +1274,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
       if (SR) ow[i] = __byte_perm(bf16_sr_sum(wn[2 * i], rnd[2 * i]), bf16_sr_sum(wn[2 * i + 1], rnd[2 * i + 1]), 0x7632);
       else ow[i] = bf16x2_rn(wn[2 * i], wn[2 * i + 1]);
     }
-    put_bf16(ow, x.d.w, e0, valid, x.vec);
+    put_bf16(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
   } else {
     uint32_t ow[2] = {0u, 0u};
 #pragma unroll
@@ -1229,11 +1283,11 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
       if (j < valid && wb < 0x7F800000u) amax_bits = max(amax_bits, wb);
       ow[j >> 2] |= e4m3_encode<SR>(__fmul_rn(wn[j], x.enc_scale), SR ? rnd[j] : 0u) << (8 * (j & 3));
     }
-    put_e4m3(ow, x.d.w, e0, valid, x.vec);
-    if (x.cc) put_compute(ow, x.cc_scale, x.cc, e0, valid, x.vec);
+    put_e4m3(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
+    if (x.cc) put_compute(ow, x.cc_scale, x.cc, e0, valid, STAGED || (x.vec & kVecCc) != 0u);
   }
   }
-  put_moments<MD>(x, e0, valid, m, v, ve);
+  put_moments<MD, STAGED>(x, e0, valid, m, v, ve);
 }
 
 // One group of a partial tile, or of a tensor whose arrays are not all staged
@@ -1398,11 +1452,11 @@ __device__ __forceinline__ void finish_block(const StepArgs& a, const TensorCtx&
     for (int j = 0; j < kGroup; ++j)
       ow[j >> 2] |= e4m3_encode<SR>(__fmul_rn(wn[j], enc), SR ? rnd[j] : 0u) << (8 * (j & 3));
   }
-  put_e4m3(ow, x.d.w, e0, valid, x.vec);
+  put_e4m3(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
   const uint32_t h_new = fp16_pow2_bits(k_new);
   if ((threadIdx.x & 3) == 0 && valid > 0) static_cast<uint16_t*>(x.scale)[e0 / kBlock] = static_cast<uint16_t>(h_new);
-  if (x.cc) put_compute(ow, fp16_value(h_new), x.cc, e0, valid, x.vec);
-  put_moments<MD>(x, e0, valid, m, v, ve);
+  if (x.cc) put_compute(ow, fp16_value(h_new), x.cc, e0, valid, STAGED || (x.vec & kVecCc) != 0u);
+  put_moments<MD, STAGED>(x, e0, valid, m, v, ve);
 }
 
 // One group of a partial tile, or of a tensor whose arrays are not all
@@ -1658,7 +1712,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
         if ((vmask >> (2 * i + 1)) & 1u) am = fmaxf(am, fabsf(wf[2 * i + 1]));
       }
     }
-    if constexpr (SRC != kExactRegs) put_moments<MD>(x, e0, valid, m, v, ve);
+    if constexpr (SRC != kExactRegs) put_moments<MD, true>(x, e0, valid, m, v, ve);
     const float et = -nt;
     const uint32_t bad = cert_not_finite(fin) ? vmask : 0u;
     const float lo_t = bad ? 0.0f : fmaxf(__fsub_rd(am, et), 0.0f);
@@ -1767,7 +1821,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
         }
       }
     }
-    if constexpr (SRC == kExactRegs) put_moments<MD>(x, e0, valid, m, v, ve);
+    if constexpr (SRC == kExactRegs) put_moments<MD, false>(x, e0, valid, m, v, ve);
   } else {
     float wn[8];
     uint32_t amx = 0u;
@@ -1786,9 +1840,9 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
       packed |= (e2m1_encode<SR>(__fdiv_rn(wn[j], d), SR ? rnd[j] : 0u) & 0xFu) << (4 * j);
-    put_moments<MD>(x, e0, valid, m, v, ve);
+    put_moments<MD, SRC != kExactRegs>(x, e0, valid, m, v, ve);
   }
-  put_fp4(packed, x.d.w, e0, valid, x.vec);
+  put_fp4(packed, x.d.w, e0, valid, SRC != kExactRegs || (x.vec & kVecW) != 0u);
   if ((threadIdx.x & 1) == 0 && valid > 0) static_cast<uint8_t*>(x.scale)[e0 / kFp4Block] = static_cast<uint8_t>(c_new);
   if (x.cc) {
     float q[8];
@@ -1796,7 +1850,7 @@ __device__ __forceinline__ void finish_fp4(const StepArgs& a, const TensorCtx& x
     uint32_t o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) o[i] = bf16x2_rn(__fmul_rn(q[2 * i], d), __fmul_rn(q[2 * i + 1], d));
-    put_bf16(o, x.cc, e0, valid, x.vec);
+    put_bf16(o, x.cc, e0, valid, SRC != kExactRegs || (x.vec & kVecCc) != 0u);
   }
 }
 

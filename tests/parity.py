@@ -72,12 +72,13 @@ def canary_damage(guards) -> int:
     return bad
 
 
-def device_copy(mt: W.Materialized, layout: str = "separate", misalign: int = 0) -> Dict[str, list]:
+def device_copy(mt: W.Materialized, layout: str = "separate", misalign=0) -> Dict[str, list]:
     """Copy a CPU-materialised workload to cuda:0.  Separately allocated
     arrays sit between canary bytes (checked by canary_damage(out["_guards"]));
     misalign > 0 also shifts every tensor by that many elements (vector path
-    off)."""
+    off), a dict the arrays that it names."""
     out = {"_guards": []}
+    shift = misalign if isinstance(misalign, dict) else dict.fromkeys(("w", "g", "m", "v", "ve", "bscale", "cc"), misalign)
     for key in ("w", "g", "m", "v", "ve"):
         src = getattr(mt, key)
         if layout == "flat" and key in mt.flat:
@@ -87,7 +88,7 @@ def device_copy(mt: W.Materialized, layout: str = "separate", misalign: int = 0)
         else:
             views = []
             for t in src:
-                v, guard = _guarded(t, misalign)
+                v, guard = _guarded(t, shift.get(key, 0))
                 out["_guards"].append(guard)
                 views.append(v)
             out[key] = views
@@ -97,7 +98,7 @@ def device_copy(mt: W.Materialized, layout: str = "separate", misalign: int = 0)
             if t is None:
                 views.append(None)
             else:
-                v, guard = _guarded(t, misalign)
+                v, guard = _guarded(t, shift.get(key, 0))
                 out["_guards"].append(guard)
                 views.append(v)
         out[key] = views
@@ -138,7 +139,7 @@ class Run:
     """A GPU optimizer and an oracle twin over the same workload."""
 
     def __init__(self, wl: W.Workload, *, warm: bool = False, layout: str = "separate",
-                 misalign: int = 0, hp: Optional[Dict] = None, mt: Optional[W.Materialized] = None):
+                 misalign=0, hp: Optional[Dict] = None, mt: Optional[W.Materialized] = None):
         self.wl = wl
         self.hp = dict(hp or {})
         self.mt = mt if mt is not None else W.materialize(wl, "cpu", layout=layout, warm_state=warm)
