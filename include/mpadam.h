@@ -296,6 +296,14 @@ int32_t mpadam_debug_tile_schedule(const int64_t* numel, int32_t n, int32_t ctas
                                    int32_t chunk_tiles, int64_t* cta_runs, int32_t* cta_first,
                                    int64_t* pool, int32_t pool_cap, int32_t* pool_count);
 
+/* Host only, no GPU: how mpadam_step deals out the tiles of a format group of
+ * `tiles` tiles in `tensors` tensors on `ctas` CTAs until mpadam_set_tail_pool
+ * is called: rule[0] = static_q, rule[1] = chunk_tiles (no pool when static_q
+ * is 1024), rule[2] = 1 when chunks are found without a table.  Errors:
+ * EINVAL. */
+int32_t mpadam_debug_pool_rule(int64_t tiles, int32_t tensors, int32_t ctas, int32_t weight_dtype,
+                               int32_t moment_dtype, int32_t* rule);
+
 /* Host only, no GPU: the shared-memory ring of the step kernel for cfg's
  * formats (weight_dtype may be any of the four) in a block of smem_bytes
  * bytes; misaligned != 0: of the instance for misaligned gradients or
@@ -334,7 +342,9 @@ int32_t mpadam_launch_info(const mpadam_state* s, int32_t* ctas, int32_t* thread
  * Until this is called the library chooses by tiles per CTA: fewer than 8
  * keep static runs (with a tile or two per CTA the pool's first claimants
  * would take several chunks each), then 768 and 4 below 16, 256 and 1 below
- * 128, and 0 and 2 above (0 and 1 for binary32 moments and long tensors).  Results do not depend on any of this.
+ * 128, and 0 and 2 above (0 and 1 for binary32 moments and long tensors);
+ * E4M3 with a scale per tensor keeps more static where tensors are many.
+ * Results do not depend on any of this.
  * Synchronises the device.  The host-buffer entry point always uses static
  * runs; the allocation-free one chooses as above.
  * Errors: EINVAL (static_q outside [0, 1024], chunk_tiles outside

@@ -27,7 +27,7 @@ EXPORTED = ["mpadam_create", "mpadam_create_ex", "mpadam_fp8_init", "mpadam_step
             "mpadam_set_tail_pool", "mpadam_launch_info", "mpadam_rng_lanes", "mpadam_step_noalloc", "mpadam_noalloc_status", "mpadam_device_status",
             "mpadam_toy_create", "mpadam_toy_step", "mpadam_toy_run", "mpadam_toy_status", "mpadam_toy_destroy",
             "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation",
-            "mpadam_debug_tile_schedule", "mpadam_debug_ring_layout"]
+            "mpadam_debug_tile_schedule", "mpadam_debug_pool_rule", "mpadam_debug_ring_layout"]
 
 
 class MPAdamError(RuntimeError):
@@ -128,6 +128,7 @@ def lib() -> ctypes.CDLL:
             "mpadam_host_buffer_free": [P, i64],
             "mpadam_debug_fail_allocation": [i32],
             "mpadam_debug_tile_schedule": [P, i32, i32, i32, i32, P, P, P, i32, P],
+            "mpadam_debug_pool_rule": [i64, i32, i32, i32, i32, P],
             "mpadam_debug_ring_layout": [P, i32, i32, P],
         }
         for name, args in sig.items():
@@ -338,6 +339,13 @@ def mpadam_debug_tile_schedule(numel, ctas: int, static_q: int, chunk_tiles: int
             continue
         _check(rc)
         return runs, first, pool[:count.value]
+
+
+def mpadam_debug_pool_rule(tiles: int, tensors: int, ctas: int, weight_dtype: int, moment_dtype: int) -> tuple:
+    """How a launch deals out its tiles by default: (static_q, chunk_tiles, whether chunks are found without a table)."""
+    out = (ctypes.c_int32 * 3)()
+    _check(lib().mpadam_debug_pool_rule(tiles, tensors, ctas, weight_dtype, moment_dtype, out))
+    return out[0], out[1], bool(out[2])
 
 
 def mpadam_debug_ring_layout(cfg: mpadam_config, misaligned: bool, smem_bytes: int) -> dict:

@@ -513,25 +513,46 @@ int32_t upload_pool(Group& g, int32_t grid, int32_t q, int32_t chunk) {
 // finds the tensor by search from the one it has (a few steps; 20,000 tensors
 // of 71 tiles on average, most of them short: 23.9 ms by search, 22.9 with the
 // table, 23.5 with 3/4 static).
+//
+// E4M3 with a scale per tensor takes less from the pool where that would lead
+// every CTA through many tensors.  A step needs each tensor's exact maximum,
+// so a warp that enters a tensor, with no maximum of its own yet, recomputes
+// the elements that might be it; static runs have about tensors + CTAs such
+// entries, the pool tensors x CTAs.  With stochastic rounding, by the rule
+// above and so:
+//   BF16 moments (bound by issue), fewer than kPoolE4m3Tiles tiles of a tensor
+//   per CTA on average: 3/4, 4 tiles (217 M parameters in 39 tensors of 9
+//   tiles a CTA 859 -> 793 us; GPT-2's shapes 447 -> 382; 4000 ragged tensors
+//   425 -> 348; at 53 tiles a CTA the two differ by 2 %, either way by
+//   rounding; a list of one tensor has no other to enter);
+//   binary32 moments hide most of it behind memory: 3/4, 4 tiles for short
+//   tensors (4000 ragged ones 433 -> 382), 1/4, 1 tile below 4 tiles of a
+//   tensor per CTA (134 M in 75 tensors 565 -> 546, GPT-2's shapes 512 -> 503;
+//   838 M in 292 tensors of 5 tiles a CTA 2148 and 2149).
 constexpr int64_t kPoolMinTilesPerCta = 8, kPoolFineTilesPerCta = 16, kPoolAllTilesPerCta = 128;
-constexpr int64_t kPoolSearchTiles = 128;
+constexpr int64_t kPoolSearchTiles = 128, kPoolE4m3Tiles = 32, kPoolE4m3TilesF32 = 4;
 
 struct PoolRule {
   int32_t static_q = 1024, chunk = 4;  // static share in 1/1024 (1024: no pool), tiles per chunk
   bool search = false;                 // no table (static_q 0)
 };
 
-PoolRule pool_rule(int64_t tiles, int32_t tensors, int32_t grid, int32_t moment_dtype) {
+PoolRule pool_rule(int64_t tiles, int32_t tensors, int32_t grid, int32_t weight_dtype, int32_t moment_dtype) {
   PoolRule r;
   if (tiles < kPoolMinTilesPerCta * grid || tiles >= INT32_MAX) return r;
-  if (tiles < kPoolFineTilesPerCta * grid) {
+  const bool e4m3 = weight_dtype == MPADAM_E4M3;
+  const bool short_tensors = tiles < kPoolSearchTiles * tensors;
+  if (tiles < kPoolFineTilesPerCta * grid ||
+      (e4m3 && (moment_dtype == MPADAM_BF16 ? tiles < kPoolE4m3Tiles * grid * (tensors - 1)
+                                            : tiles >= kPoolAllTilesPerCta * grid && short_tensors))) {
     r.static_q = 768;
-  } else if (tiles < kPoolAllTilesPerCta * grid) {
+  } else if (tiles < kPoolAllTilesPerCta * grid ||
+             (e4m3 && moment_dtype == MPADAM_F32 && tiles < kPoolE4m3TilesF32 * grid * (tensors - 1))) {
     r.static_q = 256;
     r.chunk = 1;
   } else {
     r.static_q = 0;
-    r.search = tiles >= kPoolSearchTiles * tensors;
+    r.search = !short_tensors;
     r.chunk = r.search && moment_dtype == MPADAM_F32 ? 1 : 2;
   }
   return r;
@@ -539,7 +560,7 @@ PoolRule pool_rule(int64_t tiles, int32_t tensors, int32_t grid, int32_t moment_
 
 // The group's pool for its grid: as set by the caller, else by the rule.
 int32_t setup_pool(mpadam_state* s, Group& g) {
-  PoolRule r = pool_rule(g.tiles, g.count, g.grid, s->cfg.moment_dtype);
+  PoolRule r = pool_rule(g.tiles, g.count, g.grid, g.wd, s->cfg.moment_dtype);
   if (s->pool_set) r = PoolRule{s->pool_q, s->pool_chunk, false};
   g.static_q = r.static_q;
   g.pool_len = 0;
@@ -1372,7 +1393,7 @@ extern "C" int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, 
   // (a search per chunk would cost more) a quarter, 4 tiles at a time (465 M
   // parameters in BF16: 1407 us per step with static ranges, 1208 with the pool).
   int64_t split = total_tiles;
-  PoolRule rule = pool_rule(total_tiles, n, grid, cfg->moment_dtype);
+  PoolRule rule = pool_rule(total_tiles, n, grid, cfg->weight_dtype, cfg->moment_dtype);
   if (rule.static_q < 1024) {
     if (total_tiles < kPoolSearchTiles * n) rule = PoolRule{768, 4, true};
     split = total_tiles * rule.static_q / 1024;
@@ -1631,6 +1652,21 @@ extern "C" int32_t mpadam_host_buffer_free(void* ptr, int64_t bytes) {
 extern "C" int32_t mpadam_debug_fail_allocation(int32_t after) {
   if (after < -1) return fail(MPADAM_EINVAL, "after must be >= -1");
   g_fail_countdown.store(after);
+  return MPADAM_OK;
+}
+
+extern "C" int32_t mpadam_debug_pool_rule(int64_t tiles, int32_t tensors, int32_t ctas, int32_t weight_dtype,
+                                          int32_t moment_dtype, int32_t* rule) {
+  if (tiles < 0 || tensors < 0 || ctas < 1 || ctas > (1 << 20) || !rule)
+    return fail(MPADAM_EINVAL, "tiles or tensors < 0, ctas outside [1, 2^20], or rule is NULL");
+  if (weight_dtype < MPADAM_BF16 || weight_dtype > MPADAM_NVFP4)
+    return fail(MPADAM_EINVAL, "weight_dtype must be MPADAM_BF16, MPADAM_E4M3, MPADAM_E4M3_B32 or MPADAM_NVFP4");
+  if (moment_dtype != MPADAM_F32 && moment_dtype != MPADAM_BF16)
+    return fail(MPADAM_EINVAL, "moment_dtype must be MPADAM_F32 or MPADAM_BF16");
+  const PoolRule r = pool_rule(tiles, tensors, ctas, weight_dtype, moment_dtype);
+  rule[0] = r.static_q;
+  rule[1] = r.chunk;
+  rule[2] = r.search ? 1 : 0;
   return MPADAM_OK;
 }
 
