@@ -282,6 +282,14 @@ int32_t mpadam_host_buffer_free(void* ptr, int64_t bytes);
  * wide.  Errors: EINVAL. */
 int32_t mpadam_debug_fail_allocation(int32_t after);
 
+/* Fault injection for tests: writes `value` into the tail pool's claim counters
+ * as launches that went wrong might leave them, of the state or (s NULL) of
+ * the current device's allocation-free steps, with the device idle.  error =
+ * 0: the counters of the last two calls, as if those had overlapped; else all
+ * of them, and the error word, as if a wait had given up.  Errors: EINVAL,
+ * ECUDA. */
+int32_t mpadam_debug_spoil_pool(mpadam_state* s, uint32_t value, int32_t error);
+
 /* Host only, no GPU: the tile schedule mpadam_step's launches walk for a list
  * of n tensors (numel, in launch order) on `ctas` CTAs with the tail pool
  * (static_q, chunk_tiles) of mpadam_set_tail_pool.  Tiles are 3840 elements,
@@ -354,7 +362,8 @@ int32_t mpadam_set_tail_pool(mpadam_state* s, int32_t static_q, int32_t chunk_ti
 /* Device-side status of the steps issued so far: synchronises the device,
  * returns in *code the error bits the step kernel recorded (0 = none; a
  * non-zero value means a bounded wait inside the kernel gave up and that
- * launch's results are incomplete) and clears them.  Errors: EINVAL, ECUDA. */
+ * launch's results are incomplete) and clears them, and the tail pool's claim
+ * counters, which such a launch may leave short.  Errors: EINVAL, ECUDA. */
 int32_t mpadam_device_status(mpadam_state* s, int32_t* code);
 
 /* Diagnostics: the random bits the step draws.  Writes into out (device,
@@ -377,12 +386,15 @@ int32_t mpadam_rng_lanes(uint64_t seed, int64_t step, int32_t weight_dtype, int6
  * until the process exits.  Limits: at most 8192 tensors (larger lists: MPADAM_EINVAL; use
  * mpadam_create).  The first call on a device looks up that array's device
  * address (set-up, once per device, with that device current); make that
- * first call before any stream capture.  Every call rewrites the array's
- * tables completely before the step kernel reads them, so calls issued to
- * one stream follow each other safely, but calls that overlap on the GPU
- * (different streams, or several host threads without ordering) race on
- * the shared array.  Results are bit-identical to mpadam_step on the same
- * inputs.  E4M3 weights use the caller's fp8_exp / fp8_amax rings exactly as
+ * first call before any stream capture.  Every call on more than four tensors
+ * rewrites the array's tables before the step kernel reads them (shorter lists
+ * travel with the launch), and every call that claims tiles from a tail pool
+ * clears the claim counter of the call after it.  So calls issued to one
+ * stream follow each other safely, but calls that overlap on the GPU
+ * (different streams, or several host threads without ordering) race on the
+ * shared array; up to three such calls spoil no later one, except replays of a
+ * graph that captured one of them.  Results are bit-identical to mpadam_step
+ * on the same inputs.  E4M3 weights use the caller's fp8_exp / fp8_amax rings exactly as
  * mpadam_step does (seed them with mpadam_fp8_init or equivalent values).
  * A bounded wait inside the step kernel that gives up (the launch's results
  * are then incomplete) sets a bit in the array's error word, which is not
@@ -396,7 +408,8 @@ int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, const void*
  * (companion of mpadam_step_noalloc; the paper has no counterpart).  Waits
  * for `stream`, returns in *code the error bits the step kernel recorded
  * since the last read (0 = none; non-zero: a bounded wait gave up and that
- * step's results are incomplete), and clears them.  The word is shared by
+ * step's results are incomplete), and clears them (when non-zero, the claim
+ * counters as well).  The word is shared by
  * every allocation-free call on the device, like the tables: issue this on
  * the stream the steps went to.  It allocates nothing (the word lives in the
  * same file-scope array).  Errors: EINVAL (code NULL), EUNSUPPORTED, ECUDA. */

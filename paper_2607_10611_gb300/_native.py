@@ -26,7 +26,7 @@ EXPORTED = ["mpadam_create", "mpadam_create_ex", "mpadam_fp8_init", "mpadam_step
             "mpadam_destroy", "mpadam_last_error", "mpadam_global_offset", "mpadam_global_length", "mpadam_set_grid",
             "mpadam_set_tail_pool", "mpadam_launch_info", "mpadam_rng_lanes", "mpadam_step_noalloc", "mpadam_noalloc_status", "mpadam_device_status",
             "mpadam_toy_create", "mpadam_toy_step", "mpadam_toy_run", "mpadam_toy_status", "mpadam_toy_destroy",
-            "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation",
+            "mpadam_host_buffer_alloc", "mpadam_host_buffer_free", "mpadam_debug_fail_allocation", "mpadam_debug_spoil_pool",
             "mpadam_debug_tile_schedule", "mpadam_debug_pool_rule", "mpadam_debug_ring_layout"]
 
 
@@ -127,6 +127,7 @@ def lib() -> ctypes.CDLL:
             "mpadam_host_buffer_alloc": [i64, P],
             "mpadam_host_buffer_free": [P, i64],
             "mpadam_debug_fail_allocation": [i32],
+            "mpadam_debug_spoil_pool": [P, ctypes.c_uint32, i32],
             "mpadam_debug_tile_schedule": [P, i32, i32, i32, i32, P, P, P, i32, P],
             "mpadam_debug_pool_rule": [i64, i32, i32, i32, i32, P],
             "mpadam_debug_ring_layout": [P, i32, i32, P],
@@ -318,6 +319,12 @@ def mpadam_debug_fail_allocation(after: int) -> None:
     """Test hook: the library's allocation after `after` more successful ones
     fails once (-1 disarms)."""
     _check(lib().mpadam_debug_fail_allocation(after))
+
+
+def mpadam_debug_spoil_pool(state: int, value: int, error: int = 0) -> None:
+    """Test hook: claim counters as overlapping calls (error: as launches that gave up) might leave them; state 0: those
+    of the allocation-free steps."""
+    _check(lib().mpadam_debug_spoil_pool(state or None, value, error))
 
 
 def mpadam_debug_tile_schedule(numel, ctas: int, static_q: int, chunk_tiles: int):

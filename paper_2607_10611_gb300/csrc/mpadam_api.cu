@@ -369,7 +369,8 @@ struct mpadam_state {
   // as set by set_tail_pool (until then: pool_rule)
   int32_t pool_q = 768, pool_chunk = 4;
   bool pool_set = false;
-  uint32_t* d_pool_next = nullptr;            // [groups] claim counters, zero between launches
+  uint32_t* d_pool_next = nullptr;            // [groups][kPoolCounters] claim counters, zero between launches
+  uint32_t pool_turn = 0;                     // of the next step
 };
 
 namespace {
@@ -402,6 +403,16 @@ void release(mpadam_state* s) {
   if (s->h_grads) cudaFreeHost(const_cast<void**>(s->h_grads));
   if (s->upload_done) cudaEventDestroy(s->upload_done);
   delete s;
+}
+
+size_t pool_counter_bytes(const mpadam_state* s) {
+  return sizeof(uint32_t) * mpadam::kPoolCounters * std::max<size_t>(1, s->groups.size());
+}
+
+// With the device idle.
+int32_t clear_pool_counters(mpadam_state* s) {
+  cudaError_t e = cudaMemset(s->d_pool_next, 0, pool_counter_bytes(s));
+  return e == cudaSuccess ? MPADAM_OK : cuda_fail(e, "clearing the tail-pool counters");
 }
 
 int64_t tiles_of(int64_t numel) { return (numel + mpadam::kTile - 1) / mpadam::kTile; }
@@ -769,14 +780,14 @@ int32_t create_state(const std::vector<TensorIn>& t, const mpadam_config* cfg, i
         dev_malloc(reinterpret_cast<void**>(&s->d_grads), sizeof(void*) * nn) != cudaSuccess ||
         (any_aux && dev_malloc(&s->d_aux, sizeof(TensorAux) * nn) != cudaSuccess) ||
         dev_malloc(&s->d_err, sizeof(int32_t)) != cudaSuccess ||
-        dev_malloc(&s->d_pool_next, sizeof(uint32_t) * std::max<size_t>(1, s->groups.size())) != cudaSuccess ||
+        dev_malloc(&s->d_pool_next, pool_counter_bytes(s)) != cudaSuccess ||
         host_malloc(reinterpret_cast<void**>(&s->h_grads), sizeof(void*) * nn) != cudaSuccess) {
       release(s);
       return fail(MPADAM_EALLOC, "allocation of the tensor tables failed");
     }
     e = cudaMemset(s->d_err, 0, sizeof(int32_t));
     if (e != cudaSuccess) { release(s); return cuda_fail(e, "clearing the error word"); }
-    e = cudaMemset(s->d_pool_next, 0, sizeof(uint32_t) * std::max<size_t>(1, s->groups.size()));
+    e = cudaMemset(s->d_pool_next, 0, pool_counter_bytes(s));
     if (e != cudaSuccess) { release(s); return cuda_fail(e, "clearing the tail-pool counters"); }
     e = cudaEventCreateWithFlags(&s->upload_done, cudaEventDisableTiming);
     if (e != cudaSuccess) { release(s); return cuda_fail(e, "cudaEventCreate"); }
@@ -845,7 +856,7 @@ cudaError_t launch_kernel(const void* kernel, int32_t grid, void** params, int32
 
 // One launch of a group's step kernel over its tiles [tile_base, tile_base + count).
 int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t stream, int64_t tile_base,
-                    int64_t count, const int32_t* cta_first, int32_t grid, uint32_t* pool_next = nullptr) {
+                    int64_t count, const int32_t* cta_first, int32_t grid, uint32_t* pool_counters = nullptr) {
   bool mis = g.w_mis;
   for (int32_t p = g.first; !mis && p < g.first + g.count; ++p)
     mis = s->numel[s->order[p]] > 0 && !is_aligned(s->h_grads[p], 16);
@@ -853,8 +864,9 @@ int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t 
   a.cta_first = cta_first;
   a.tile_base = tile_base;
   a.total_tiles = count;
-  if (pool_next && g.pool_chunks > 0) {  // whole-group launches only: the pool covers all of its tiles
-    a.pool_next = pool_next;
+  if (pool_counters && g.pool_chunks > 0) {  // whole-group launches only: the pool covers all of its tiles
+    a.pool_next = pool_counters + s->pool_turn % mpadam::kPoolCounters;
+    a.pool_clear = pool_counters + (s->pool_turn + 1) % mpadam::kPoolCounters;
     a.pool_chunks = g.pool_chunks;
     a.static_q = g.static_q;
     if (g.pool_len > 0) a.pool_len = g.pool_len;  // pool_base 0: every tile is in the pool
@@ -1002,6 +1014,8 @@ int32_t mpadam_set_grid(mpadam_state* s, int32_t ctas) {
   if (rc) return rc;
   cudaError_t e = cudaDeviceSynchronize();  // the old table may be in use
   if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
+  rc = clear_pool_counters(s);
+  if (rc) return rc;
   release_pipeline(s);  // the host-buffer pipeline's per-chunk tables follow the grid: rebuilt on next use
   for (auto& g : s->groups) {
     rc = upload_cta_table(g, ctas == 0 ? g.default_grid : ctas);
@@ -1019,6 +1033,8 @@ int32_t mpadam_set_tail_pool(mpadam_state* s, int32_t static_q, int32_t chunk_ti
   if (rc) return rc;
   cudaError_t e = cudaDeviceSynchronize();  // the old pool may be in use
   if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
+  rc = clear_pool_counters(s);
+  if (rc) return rc;
   s->pool_q = static_q;
   s->pool_chunk = chunk_tiles;
   s->pool_set = true;
@@ -1046,7 +1062,7 @@ int32_t mpadam_device_status(mpadam_state* s, int32_t* code) {
   if (e != cudaSuccess) return cuda_fail(e, "reading the error word");
   e = cudaMemset(s->d_err, 0, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
-  return MPADAM_OK;
+  return clear_pool_counters(s);
 }
 
 int32_t mpadam_step(mpadam_state* s, const void* const* grads, int64_t step, cudaStream_t stream) {
@@ -1069,9 +1085,10 @@ int32_t mpadam_step(mpadam_state* s, const void* const* grads, int64_t step, cud
   for (size_t i = 0; i < s->groups.size(); ++i) {
     const Group& g = s->groups[i];
     if (g.tiles == 0) continue;
-    rc = launch_step(s, g, step, stream, 0, g.tiles, g.d_cta_first, g.grid, s->d_pool_next + i);
+    rc = launch_step(s, g, step, stream, 0, g.tiles, g.d_cta_first, g.grid, s->d_pool_next + i * mpadam::kPoolCounters);
     if (rc) return rc;
   }
+  ++s->pool_turn;
   return MPADAM_OK;
 }
 
@@ -1274,7 +1291,7 @@ constexpr size_t kNoAllocTableBytes =
 // it, and only mpadam_noalloc_status reads and clears it.  The array starts
 // zeroed when the library's module loads.
 constexpr size_t kNoAllocErrOffset = kNoAllocTableBytes;
-// The tail pool's claim counter sits in the same slot; every launch leaves it at zero.
+// The tail pool's claim counters (kPoolCounters) sit in the same slot.
 constexpr size_t kNoAllocPoolOffset = kNoAllocTableBytes + 64;
 constexpr size_t kNoAllocScratchBytes = kNoAllocTableBytes + 256;  // 606,464 bytes
 static_assert(kNoAllocErrOffset % 256 == 0, "the error word keeps the array's alignment");
@@ -1309,6 +1326,7 @@ constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 unsigned char* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 int g_noalloc_sms[kNoAllocMaxDevices] = {};
+std::atomic<uint32_t> g_noalloc_turn[kNoAllocMaxDevices] = {};  // which claim counter comes next
 
 int32_t noalloc_setup(int dev, unsigned char** scratch, int* sms) {
   if (dev < 0 || dev >= kNoAllocMaxDevices) return fail(MPADAM_EUNSUPPORTED, "device %d beyond the set-up table", dev);
@@ -1400,7 +1418,10 @@ extern "C" int32_t mpadam_step_noalloc(const mpadam_tensor* tensors, int32_t n, 
     a.pool_base = split;
     a.pool_len = rule.chunk;
     a.pool_chunks = (int32_t)((total_tiles - split + a.pool_len - 1) / a.pool_len);
-    a.pool_next = reinterpret_cast<uint32_t*>(scratch + kNoAllocPoolOffset);
+    uint32_t* counters = reinterpret_cast<uint32_t*>(scratch + kNoAllocPoolOffset);
+    const uint32_t turn = g_noalloc_turn[dev].fetch_add(1);
+    a.pool_next = counters + turn % mpadam::kPoolCounters;
+    a.pool_clear = counters + (turn + 1) % mpadam::kPoolCounters;
   }
   a.n_desc = n;
 
@@ -1480,6 +1501,10 @@ extern "C" int32_t mpadam_noalloc_status(cudaStream_t stream, int32_t* code) {
   if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
   e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+  if (*code != 0) {  // a launch that gave up may not have claimed all that it would have
+    e = cudaMemset(scratch + kNoAllocPoolOffset, 0, sizeof(uint32_t) * mpadam::kPoolCounters);
+    if (e != cudaSuccess) return cuda_fail(e, "clearing the tail-pool counters");
+  }
   return MPADAM_OK;
 }
 
@@ -1682,6 +1707,44 @@ extern "C" int32_t mpadam_debug_ring_layout(const mpadam_config* cfg, int32_t mi
   if (rc) return rc;
   const int32_t out[8] = {g.stages, g.stage_bytes, g.off_g, g.off_m, g.off_v, g.off_ve, g.off_s, mpadam::kStaticSmem};
   std::memcpy(layout, out, sizeof out);
+  return MPADAM_OK;
+}
+
+extern "C" int32_t mpadam_debug_spoil_pool(mpadam_state* s, uint32_t value, int32_t error) {
+  int32_t rc = s ? check_device(s) : MPADAM_OK;
+  if (rc) return rc;
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
+  uint32_t *counters = nullptr, turn = 0;
+  int32_t* err = nullptr;
+  size_t sets = 1;
+  if (s) {
+    counters = s->d_pool_next;
+    err = s->d_err;
+    turn = s->pool_turn;
+    sets = s->groups.size();
+  } else {
+    int dev = -1, sms = 0;
+    unsigned char* scratch = nullptr;
+    e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    rc = noalloc_setup(dev, &scratch, &sms);
+    if (rc) return rc;
+    counters = reinterpret_cast<uint32_t*>(scratch + kNoAllocPoolOffset);
+    err = reinterpret_cast<int32_t*>(scratch + kNoAllocErrOffset);
+    turn = g_noalloc_turn[dev].load();
+  }
+  for (size_t i = 0; i < sets; ++i)
+    for (uint32_t back = 1; back <= mpadam::kPoolCounters; ++back) {
+      if (error == 0 && back > 2) continue;
+      uint32_t* c = counters + i * mpadam::kPoolCounters + (turn - back) % mpadam::kPoolCounters;
+      e = cudaMemcpy(c, &value, sizeof value, cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) return cuda_fail(e, "writing a claim counter");
+    }
+  if (error != 0) {
+    e = cudaMemcpy(err, &error, sizeof error, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "writing the error word");
+  }
   return MPADAM_OK;
 }
 

@@ -43,6 +43,11 @@ constexpr int kTile = kConsumers * kGroup;          // 3840 elements per tile (1
 constexpr int kMaxStages = 8;
 constexpr int kInlineTensors = 4;                   // launches of at most this many tensors carry their tables inline
 constexpr int kPhiloxRounds = 10;
+// Claim counters of a sequence of pooled launches, used in turn.  A launch
+// leaves its own at zero (so that a captured one can be replayed) and clears
+// the next one's, so launches that were wrongly let overlap, and that leave
+// anything in theirs, spoil no later one.
+constexpr int kPoolCounters = 4;
 constexpr int kBlock = 32;                          // elements per block scale (block-scaled E4M3)
 constexpr int kTileBlocks = kTile / kBlock;         // 120 block scales per tile (240 bytes)
 static_assert(kTile % kBlock == 0 && kBlock == 4 * kGroup, "a block is one quad of consumer threads");
@@ -142,6 +147,7 @@ struct StepArgs {
   int32_t* err;              // DeviceError bits, or nullptr
   const PoolChunk* pool;     // [pool_chunks] tail pool, or nullptr (static ranges only)
   uint32_t* pool_next;       // next unclaimed pool chunk; zero when the launch starts and again when it ends
+  uint32_t* pool_clear;      // the counter that the launch after this one claims from
   int32_t pool_chunks;       // 0: no pool
   // A pool without a table (pool == nullptr): the static ranges share tiles
   // [tile_base, pool_base), and chunk j is the pool_len tiles from pool_base + j pool_len on.

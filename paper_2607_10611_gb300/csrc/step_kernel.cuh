@@ -2021,8 +2021,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
   if (warp == kConsumerWarps) {
     if (lane != 0) return;
     // Every CTA's claims end with one beyond the pool, pool_chunks + gridDim.x
-    // in all: the last of them wraps the counter back to 0 for the next launch
-    // (a memset before every launch cost a gap of its own on the stream).
+    // in all: the last of them wraps the counter back to 0 (a memset before
+    // every launch cost a gap of its own on the stream).  A CTA that gives up
+    // makes fewer: reading the launch's status clears the counters.
     auto claim = [&]() { return atomicInc(a.pool_next, static_cast<uint32_t>(a.pool_chunks) + gridDim.x - 1u); };
     bool failed = false;
     bool ahead = false;  // a claim (j) made before the run in hand is done
@@ -2065,8 +2066,6 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
         if (!mbar_wait(smem_addr(&full_bar[it % S]), static_cast<uint32_t>((it / S) & 1)) && a.err)
           atomicOr(a.err, kErrDrainWait);
       }
-      if (pooled && !(ahead && j >= static_cast<uint32_t>(a.pool_chunks)))
-        while (claim() < static_cast<uint32_t>(a.pool_chunks)) {}  // leave the counter as a CTA that finished would
       return;
     }
     // no more work: once the next stage is free, post the end marker there
@@ -2076,6 +2075,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant
     }
     heads[ps].k = -1;
     mbar_arrive(smem_addr(&full_bar[ps]));
+    if (pooled && blockIdx.x == 0) *a.pool_clear = 0u;
     return;
   }
 
