@@ -23,19 +23,29 @@ _STORAGE = {"bf16": torch.bfloat16, "e4m3": torch.uint8, "e4m3_b32": torch.uint8
 _SCALES = {"e4m3_b32": torch.float16, "nvfp4": torch.uint8}
 
 
-def _pointers(tensors) -> array.array:
-    """Device pointers of tensors, as the array that the C ABI takes."""
-    if not isinstance(tensors, (list, tuple)):
-        tensors = list(tensors)
-    try:
-        return array.array("Q", map(torch.Tensor.data_ptr, tensors))
-    except TypeError:  # not torch tensors: anything with a data_ptr()
-        return array.array("Q", [t.data_ptr() for t in tensors])
+# The current stream's raw handle, without the Stream object (which costs 2 us); private to torch, so it may go.
+_get_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _raw_stream(device: torch.device) -> int:
-    """Handle of the device's current stream (without the Stream object, which costs 2 us)."""
-    return torch._C._cuda_getCurrentRawStream(device.index)
+    """Handle of the device's current stream."""
+    try:
+        return _get_raw_stream(device.index)
+    except TypeError:  # torch has none, or the device no index
+        return torch.cuda.current_stream(device).cuda_stream
+
+
+_PLAIN = frozenset((torch.Tensor, torch.nn.Parameter))  # types whose data_ptr is the base class's
+
+
+def _pointers(tensors) -> array.array:
+    """Device pointers of tensors, as the array that the C ABI takes (98 of them on the GPU's host: 7.6 us, 8.0 by
+    calling each one's own method)."""
+    if type(tensors) is not list:
+        tensors = list(tensors)
+    if _PLAIN.issuperset(map(type, tensors)):
+        return array.array("Q", [*map(torch.Tensor.data_ptr, tensors)])
+    return array.array("Q", [t.data_ptr() for t in tensors])  # a subclass may have its own, anything else one at all
 
 
 class HostBuffer:
