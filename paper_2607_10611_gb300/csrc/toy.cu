@@ -219,7 +219,10 @@ __global__ void toy_update_kernel(const __grid_constant__ ToyArgs a) {
 // Waits are bounded: a CTA whose wait runs out sets *a.err and returns, and so
 // do the others when theirs do.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kToySpinLimit = 1u << 20;     // polls (about a second) before a wait gives up
+#ifndef MPADAM_TOY_SPIN_LIMIT
+#define MPADAM_TOY_SPIN_LIMIT (1u << 20)
+#endif
+constexpr uint32_t kToySpinLimit = MPADAM_TOY_SPIN_LIMIT;  // polls (about a second) before a wait gives up
 constexpr unsigned long long kToyEmpty = ~0ull;  // no sum has these bits (one that would is stored as another NaN)
 
 __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {

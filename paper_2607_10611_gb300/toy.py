@@ -1,6 +1,7 @@
 """The BF16-stored matrix-fitting diagnostic (the toy diagnostic of Sec. 5.1
 and its appendix) on torch tensors: argument marshalling around
-mpadam_toy_create / mpadam_toy_step (no arithmetic here).
+mpadam_toy_create / mpadam_toy_step / mpadam_toy_run / mpadam_toy_status (no
+arithmetic here).
 """
 from __future__ import annotations
 
@@ -42,14 +43,19 @@ class ToyDiagnostic:
 
     def run(self, first_step: int, steps: int, losses: Optional[torch.Tensor] = None,
             stream: Optional[torch.cuda.Stream] = None):
-        """Steps first_step .. first_step + steps - 1 inside one kernel;
-        losses: a CUDA float64 tensor of `steps` elements, or None."""
+        """Steps first_step .. first_step + steps - 1 inside one kernel (one
+        per 8192 steps), asynchronously; losses: a CUDA float64 tensor of
+        `steps` elements, or None.  The kernel's CTAs wait on one another, each
+        wait bounded (about a second): ask device_status() before relying on
+        the results."""
         s = (stream or torch.cuda.current_stream(self.w.device)).cuda_stream
         N.mpadam_toy_run(self.state, self.w.data_ptr(), self.wstar.data_ptr(), first_step, steps,
                          losses.data_ptr() if losses is not None else 0, s)
 
     def device_status(self) -> int:
-        """Device error word of the runs so far (0 = none); synchronises."""
+        """Synchronises; device error word of the runs since the last call: 0,
+        or 1 when a wait inside a run gave up.  Then neither w nor the losses
+        nor this object's state are valid: make a new one."""
         return N.mpadam_toy_status(self.state)
 
     def close(self):
