@@ -75,3 +75,37 @@ def test_captured_steps_replay(name, pooled):
     assert a.opt.device_status() == 0
     _same(a, b)
     a.close(); b.close()
+
+
+@pytest.mark.parametrize("name,pooled", [("flat_1m", False), ("llama_1p5b_mixed", False), ("gpt2_124m", True)])
+def test_captured_behind_a_copy_and_behind_a_join(name, pooled):
+    """The work ahead of a captured step need not be a kernel: the first step of
+    a state copies its gradient table inside the capture, and the next waits
+    for gradients written on another captured stream."""
+    a, b = _pair(name, pooled)
+    base = [g.clone() for g in a.dev["g"]]
+    side = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        a.opt.step(a.dev["g"], 1)
+        main = torch.cuda.current_stream()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            for g, g0 in zip(a.dev["g"], base):
+                torch.mul(g0, 1.5, out=g)
+        main.wait_stream(side)
+        a.opt.step(a.dev["g"], 2)
+    for _ in range(2):
+        for g, g0 in zip(a.dev["g"], base):
+            g.copy_(g0)
+        graph.replay()
+    torch.cuda.synchronize()
+    for _ in range(2):
+        for t, f in ((1, 1.0), (2, 1.5)):
+            for g, g0 in zip(b.dev["g"], base):
+                torch.mul(g0, f, out=g)
+            b.opt.step(b.dev["g"], t)
+            torch.cuda.synchronize()
+    assert a.opt.device_status() == 0
+    _same(a, b)
+    a.close(); b.close()
