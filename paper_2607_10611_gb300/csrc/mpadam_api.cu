@@ -79,7 +79,8 @@ size_t weight_bytes(int32_t wd, int64_t n) {
   return wd == MPADAM_NVFP4 ? (size_t)((n + 1) / 2) : (size_t)n * elem_size(wd);
 }
 
-bool is_aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
+// a: a power of two
+bool is_aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 // Per-step binary32 scalars of the canonical update, from binary64.
 float toward_zero(double x) {
@@ -855,10 +856,12 @@ cudaError_t launch_kernel(const void* kernel, int32_t grid, void** params, int32
 }
 
 // One launch of a group's step kernel over its tiles [tile_base, tile_base + count).
+// grads_off: whether some gradients of the list are not 16-byte aligned.
 int32_t launch_step(mpadam_state* s, const Group& g, int64_t step, cudaStream_t stream, int64_t tile_base,
-                    int64_t count, const int32_t* cta_first, int32_t grid, uint32_t* pool_counters = nullptr) {
+                    int64_t count, const int32_t* cta_first, int32_t grid, bool grads_off = false,
+                    uint32_t* pool_counters = nullptr) {
   bool mis = g.w_mis;
-  for (int32_t p = g.first; !mis && p < g.first + g.count; ++p)
+  for (int32_t p = g.first; grads_off && !mis && p < g.first + g.count; ++p)
     mis = s->numel[s->order[p]] > 0 && !is_aligned(s->h_grads[p], 16);
   StepArgs a = base_args(s, g, mis);
   a.cta_first = cta_first;
@@ -1073,10 +1076,12 @@ int32_t mpadam_step(mpadam_state* s, const void* const* grads, int64_t step, cud
   if (s->n == 0 || tiles == 0) return MPADAM_OK;
   if (!grads) return fail(MPADAM_EINVAL, "grads is NULL");
   const size_t gsz = elem_size(s->cfg.grad_dtype);
+  uintptr_t any = 0;
   for (int32_t k = 0; k < s->n; ++k) {
     if (s->numel[k] == 0) continue;
     if (!grads[k]) return fail(MPADAM_EINVAL, "grads[%d] is NULL", k);
     if (!is_aligned(grads[k], gsz)) return fail(MPADAM_EINVAL, "grads[%d] not aligned to its element size", k);
+    any |= reinterpret_cast<uintptr_t>(grads[k]);
   }
   int32_t rc = check_device(s);
   if (rc) return rc;
@@ -1085,7 +1090,8 @@ int32_t mpadam_step(mpadam_state* s, const void* const* grads, int64_t step, cud
   for (size_t i = 0; i < s->groups.size(); ++i) {
     const Group& g = s->groups[i];
     if (g.tiles == 0) continue;
-    rc = launch_step(s, g, step, stream, 0, g.tiles, g.d_cta_first, g.grid, s->d_pool_next + i * mpadam::kPoolCounters);
+    rc = launch_step(s, g, step, stream, 0, g.tiles, g.d_cta_first, g.grid, any % 16 != 0,
+                     s->d_pool_next + i * mpadam::kPoolCounters);
     if (rc) return rc;
   }
   ++s->pool_turn;
