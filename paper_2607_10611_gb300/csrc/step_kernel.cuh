@@ -4,10 +4,10 @@
 // (one per SM) is a producer/consumer pipeline over its tiles:
 //   - one producer warp (one elected lane) picks each tile -- the next of its
 //     own range, then chunks claimed from the launch's tail pool -- posts the
-//     tile and what is needed of its tensor beside the stage, and streams the tile's slice of
-//     every array (weights w, gradients g and the moments mu, nu, nu_e, each
-//     one contiguous run of bytes) into a multi-stage shared-memory ring with
-//     1-D TMA bulk copies (cp.async.bulk ... mbarrier::complete_tx), evict-
+//     tile and what is needed of its tensor beside the stage, and streams the
+//     tile's slice of every array (weights w, gradients g and the moments mu,
+//     nu, nu_e, each one contiguous run of bytes) into a multi-stage
+//     shared-memory ring with 1-D TMA bulk copies (cp.async.bulk ... mbarrier::complete_tx), evict-
 //     first in L2 since every byte is used once; an end marker in the next
 //     stage tells the consumers that the work is done;
 //   - fifteen consumer warps wait on the stage's mbarrier, read their 8
@@ -17,10 +17,11 @@
 //     Philox4x32-10 bits) and store w, mu, nu, nu_e straight back to HBM with
 //     vector stores (256-bit for binary32 arrays), then release the stage.
 // Memory latency is hidden by the ring, not by occupancy, so the consumers'
-// instruction stream is the only other limit.  A tensor's last bytes
-// that are not a whole 16-byte line, and tensors with misaligned weights or
-// moments, are read by the consumers directly from global memory with the
-// same arithmetic; misaligned gradients go through the ring all the same.  No tensor cores: nothing here is a contraction.
+// instruction stream is the only other limit.  A tensor's last bytes that are
+// not a whole 16-byte line, and arrays of misaligned weights or moments, are
+// read by the consumers directly from global memory with the same arithmetic;
+// misaligned gradients (of NVFP4 lists excepted) go through the ring all the
+// same.  No tensor cores: nothing here is a contraction.
 //
 // Numerics: every floating-point operation of the canonical sequence is an
 // explicit round-to-nearest intrinsic (__fmul_rn, __fadd_rn, __fmaf_rn,
@@ -220,11 +221,11 @@ __device__ __forceinline__ Upd madam_update(const StepScalars& s, float w, float
 // are by memory wherever an element has few bytes (BF16 moments, FP8 and FP4
 // weights).  With the packed update, the packed encoders and the tighter
 // bound below, instructions per element went from 84 to 61 (BF16 weights and
-// moments, SR) and from 115 to 83 (E4M3, SR); a 217 M-parameter list with BF16
-// moments went from 984 to 670 us (E4M3, nearest), 1135 to 880 (E4M3, SR),
-// 993 to 768 and 1085 to 911 (block-scaled E4M3), 867 to 804 and 1142 to 1048
-// (NVFP4); with binary32 moments NVFP4 with SR 1272 to 1225 us, E4M3 1152 to
-// 1099 (the others are bound by memory).
+// moments, SR) and from 115 to 82 (E4M3, SR).  A 217 M-parameter list with
+// BF16 moments, nearest and SR, before all this and at present: E4M3 983 ->
+// 644 us and 1135 -> 822, block-scaled E4M3 991 -> 740 and 1083 -> 896, NVFP4
+// 865 -> 778 and 1141 -> 946; with binary32 moments, where memory is the
+// bound, NVFP4 with SR 1274 -> 1167 us and E4M3 1152 -> 1071.
 // ---------------------------------------------------------------------------
 using f32x2 = uint64_t;  // low half: the even element
 
@@ -626,8 +627,8 @@ __device__ __forceinline__ uint32_t staged_bytes(const void* base, int count, in
 // reducer's bucket packs gradients without padding; a flat buffer puts tensors
 // at multiples of 8 elements).  A launch with any such array runs the MIS
 // instance of the kernel (read element by element, a list of 4000 ragged
-// tensors in BF16 took 655 us with its gradients in a bucket, now 395; E4M3
-// with BF16 moments in a flat buffer 752, now 374).  It is an instance of its
+// tensors in BF16 took 651 us with its gradients in a bucket, now 384; E4M3
+// with BF16 moments in a flat buffer 1096, now 361).  It is an instance of its
 // own because its code, though skipped for aligned arrays, slowed short
 // launches by 3 to 7 % and NVFP4 with SR by 4 %; NVFP4 has none and reads them
 // in the element-wise path.  Such an array keeps its place modulo 16 in its
@@ -1522,8 +1523,6 @@ __device__ __forceinline__ uint32_t e2m1_encode(float x, uint32_t r) {
   return x != x ? 0u : code;
 }
 
-// Eight binary32 -> packed E2M1 codes, nearest-even with saturation at +-6
-// (the hardware conversion; used only on finite values).
 // Two binary32 -> two E2M1 codes, nearest-even (hardware conversion; x0 in
 // the low nibble).
 __device__ __forceinline__ uint32_t e2m1x2_rn(float x0, float x1) {

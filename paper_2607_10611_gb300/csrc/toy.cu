@@ -205,11 +205,11 @@ __global__ void toy_update_kernel(const __grid_constant__ ToyArgs a) {
 //      and final counts.
 // Each CTA waits on a 128-byte line of its own: with every CTA polling the
 // slots, a few lines of one L2 slice, a step took 8.9 us (8.0 so).  What
-// bounds it now are the scattered accesses over three arrays of 168 MB together
-// and the two exchanges: with all of them in L2 (1 Mi entries) a step is about
-// a third shorter.  Slots alternate between two buffers, emptied by
-// their one reader.  Publishing needs no fence: the slot's value depends on the
-// reads that have to come first.
+// bounds it now are the scattered accesses over four arrays of 235 MB together
+// (weights, targets and two of hit counts) and the two exchanges: with all of
+// them in L2 (1 Mi entries) a step is about a third shorter.  Slots alternate
+// between two buffers, emptied by their one reader.  Publishing needs no
+// fence: the slot's value depends on the reads that have to come first.
 //
 // binary64 runs at half a lane per cycle and scheduler here (a warp
 // instruction holds the unit for 64 cycles), so the squares are formed with

@@ -1,7 +1,9 @@
-"""The hardware approximations behind the step kernel's certified fast path
-(sqrt.approx.f32, div.approx.f32) stay far inside the 2^-19 relative error
-the certificate assumes, over operands spanning the ranges the update sees
-(denominators in [2^-125, 2^125], numerators of any magnitude)."""
+"""The step kernel's hardware approximations: sqrt.approx.ftz.f32 stays inside
+the 2^-21 relative error that the certified fast path assumes (its other
+approximation, the reciprocal, is measured in test_gpu_cert.py), and
+div.approx.f32, the start of the NVFP4 scale search, is as close, over operands
+spanning the ranges the update sees (divisors in [2^-125, 2^125], numerators
+of any magnitude)."""
 import ctypes
 import subprocess
 from pathlib import Path

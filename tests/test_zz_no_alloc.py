@@ -10,7 +10,7 @@ gave up (that word lives in the same array).
 
 Lists covered: more tensors than one table-fill launch carries (384), the
 E4M3 and BF16-moment formats, empty tensors passed with NULL pointers, and
-exactly the 8192-tensor limit.  The per-CTA table's own limit (4096 CTAs) is
+exactly the 8192-tensor limit.  The grid's own limit (1024 CTAs) is
 not reachable here: the step kernel runs one CTA per SM.
 
 The file name makes pytest collect it last, so a failure here leaves every
