@@ -212,7 +212,9 @@ def mpadam_fp8_init(state: int, init_exp: Sequence[int], first_step: int, stream
 def mpadam_step(state: int, grads: Sequence[int], step: int, stream: int = 0) -> None:
     """grads: one pointer per tensor; an array.array("Q") of them is passed as it is."""
     arr = grads if type(grads) is array.array and grads.typecode == "Q" else _ptr_array(grads)
-    _check(lib().mpadam_step(state, arr.buffer_info()[0], step, stream or None))
+    status = lib().mpadam_step(state, arr.buffer_info()[0], step, stream or None)
+    if status:
+        _check(status)
 
 
 def mpadam_step_host(state: int, host_grads: Sequence[int], host_w_out: Sequence[int], step: int,

@@ -35,17 +35,33 @@ def _raw_stream(device: torch.device) -> int:
         return torch.cuda.current_stream(device).cuda_stream
 
 
+_data_ptr = torch.Tensor.data_ptr
 _PLAIN = frozenset((torch.Tensor, torch.nn.Parameter))  # types whose data_ptr is the base class's
+_MANY = 170  # tensors; a look at that many types takes as long as one at the classes, about 1.9 us
+
+
+def _own_data_ptr() -> bool:
+    """Whether a subclass of Tensor that is loaded has a data_ptr of its own."""
+    classes = torch.Tensor.__subclasses__()
+    for c in classes:
+        if c.data_ptr is not _data_ptr:
+            return True
+        classes += c.__subclasses__()
+    return False
 
 
 def _pointers(tensors) -> array.array:
-    """Device pointers of tensors, as the array that the C ABI takes (98 of them on the GPU's host: 7.6 us, 8.0 by
-    calling each one's own method)."""
+    """Device pointers of tensors, as the array that the C ABI takes.  The base class's data_ptr, called on all of them
+    by map, is a quarter faster than each one's own, and right where no tensor has its own (98 tensors on the GPU's
+    host: 7.6 us with the look at their types, 8.0 by each one's own; a step of 4000 tensors 272 us and 338)."""
     if type(tensors) is not list:
         tensors = list(tensors)
-    if _PLAIN.issuperset(map(type, tensors)):
-        return array.array("Q", [*map(torch.Tensor.data_ptr, tensors)])
-    return array.array("Q", [t.data_ptr() for t in tensors])  # a subclass may have its own, anything else one at all
+    if _PLAIN.issuperset(map(type, tensors)) if len(tensors) < _MANY else not _own_data_ptr():
+        try:
+            return array.array("Q", [*map(_data_ptr, tensors)])
+        except TypeError:  # not torch tensors: anything with a data_ptr()
+            pass
+    return array.array("Q", [t.data_ptr() for t in tensors])
 
 
 class HostBuffer:

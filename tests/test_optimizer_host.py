@@ -1,6 +1,7 @@
 """What MPAdam.step hands to the C ABI, checked on the host (no GPU): each
 gradient's own data_ptr(), whatever kind of object it is, and the current
 stream, also where torch does not offer its raw handle."""
+import gc
 import types
 
 import pytest
@@ -25,21 +26,32 @@ def step(monkeypatch):
     return run
 
 
-class Moved(torch.Tensor):
-    """A tensor whose data lies elsewhere."""
+def _moved(mixin):
+    """A kind of tensor whose data lies elsewhere: its own method, or one from another base."""
+    class Elsewhere:
+        def data_ptr(self):
+            return 0x7000
+    if mixin:
+        return type("Moved", (Elsewhere, torch.Tensor), {})
+    return type("Moved", (torch.Tensor,), {"data_ptr": Elsewhere.data_ptr})
 
-    def data_ptr(self):
-        return 0x7000
 
-
-def test_pointers_of_every_kind_of_gradient(step):
+@pytest.mark.parametrize("n", [1, 2 * O._MANY])  # by the tensors' types, and by the classes that are loaded
+@pytest.mark.parametrize("mixin", [False, True])
+def test_pointers_of_every_kind_of_gradient(step, mixin, n):
+    gc.collect()  # classes of earlier tests
+    assert not O._own_data_ptr()
     a, b = torch.zeros(3), torch.nn.Parameter(torch.zeros(5))
-    c, d = torch.zeros(2).as_subclass(Moved), types.SimpleNamespace(data_ptr=lambda: 0x9000)
+    d = types.SimpleNamespace(data_ptr=lambda: 0x9000)
+    assert step([a, b] * n)[0] == [a.data_ptr(), b.data_ptr()] * n
+    assert step([a, d] * n)[0] == [a.data_ptr(), 0x9000] * n
+    c = torch.zeros(2).as_subclass(_moved(mixin))
+    assert O._own_data_ptr()
     want = [a.data_ptr(), b.data_ptr(), 0x7000, 0x9000]
-    for grads in ([a, b, c, d], (a, b, c, d), (x for x in (a, b, c, d))):
-        assert step(grads)[0] == want
+    for grads in ([a, b, c, d] * n, (a, b, c, d) * n, (x for x in [a, b, c, d] * n)):
+        assert step(grads)[0] == want * n
     with pytest.raises(AttributeError):
-        step([a, None])
+        step([a, None] * n)
 
 
 def test_current_stream(step, monkeypatch):
