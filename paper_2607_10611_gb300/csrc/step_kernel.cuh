@@ -7,9 +7,9 @@
 //     tile and what is needed of its tensor beside the stage, and streams the
 //     tile's slice of every array (weights w, gradients g and the moments mu,
 //     nu, nu_e, each one contiguous run of bytes) into a multi-stage
-//     shared-memory ring with 1-D TMA bulk copies (cp.async.bulk ... mbarrier::complete_tx), evict-
-//     first in L2 since every byte is used once; an end marker in the next
-//     stage tells the consumers that the work is done;
+//     shared-memory ring with 1-D TMA bulk copies (cp.async.bulk ...
+//     mbarrier::complete_tx), evict-first in L2 since every byte is used once;
+//     an end marker in the next stage tells the consumers that the work is done;
 //   - fifteen consumer warps wait on the stage's mbarrier, read their 8
 //     elements from shared memory, run the canonical binary32 update
 //     (Algorithm 1 with the Algorithm 2 options, arxiv 2607.10611), round the
@@ -220,8 +220,8 @@ __device__ __forceinline__ Upd madam_update(const StepScalars& s, float w, float
 // slots.  The step's instances are bound by instruction issue before they
 // are by memory wherever an element has few bytes (BF16 moments, FP8 and FP4
 // weights).  With the packed update, the packed encoders and the tighter
-// bound below, instructions per element went from 84 to 61 (BF16 weights and
-// moments, SR) and from 115 to 82 (E4M3, SR).  A 217 M-parameter list with
+// bound below, instructions per element went from 84 to 59 (BF16 weights and
+// moments, SR) and from 115 to 78 (E4M3, SR).  A 217 M-parameter list with
 // BF16 moments, nearest and SR, before all this and at present: E4M3 983 ->
 // 644 us and 1135 -> 822, block-scaled E4M3 991 -> 740 and 1083 -> 896, NVFP4
 // 865 -> 778 and 1141 -> 946; with binary32 moments, where memory is the
