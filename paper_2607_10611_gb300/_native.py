@@ -151,6 +151,10 @@ def _check(status: int) -> None:
         raise MPAdamError(status, mpadam_last_error())
 
 
+# Type code of arrays of 64-bit words: unsigned long where it has 64 bits (98 pointers go in in 0.7 us, as "Q" in 1.1).
+WORD = "L" if array.array("L").itemsize == 8 else "Q"
+
+
 def _ptr_array(ptrs: Iterable[int]) -> array.array:
     """Pointers (ints; None = NULL) as 64-bit words; pass buffer_info()[0] while the array lives."""
     ptrs = list(ptrs)
@@ -210,8 +214,8 @@ def mpadam_fp8_init(state: int, init_exp: Sequence[int], first_step: int, stream
 
 
 def mpadam_step(state: int, grads: Sequence[int], step: int, stream: int = 0) -> None:
-    """grads: one pointer per tensor; an array.array("Q") of them is passed as it is."""
-    arr = grads if type(grads) is array.array and grads.typecode == "Q" else _ptr_array(grads)
+    """grads: one pointer per tensor; an array.array of 64-bit words ("Q" or WORD) is passed as it is."""
+    arr = grads if type(grads) is array.array and grads.typecode in ("Q", WORD) else _ptr_array(grads)
     status = lib().mpadam_step(state, arr.buffer_info()[0], step, stream or None)
     if status:
         _check(status)

@@ -53,15 +53,15 @@ def _own_data_ptr() -> bool:
 def _pointers(tensors) -> array.array:
     """Device pointers of tensors, as the array that the C ABI takes.  The base class's data_ptr, called on all of them
     by map, is a quarter faster than each one's own, and right where no tensor has its own (98 tensors on the GPU's
-    host: 7.6 us with the look at their types, 8.0 by each one's own; a step of 4000 tensors 272 us and 338)."""
+    host: 7.1 us with the look at their types, 7.6 by each one's own)."""
     if type(tensors) is not list:
         tensors = list(tensors)
     if _PLAIN.issuperset(map(type, tensors)) if len(tensors) < _MANY else not _own_data_ptr():
         try:
-            return array.array("Q", [*map(_data_ptr, tensors)])
+            return array.array(N.WORD, [*map(_data_ptr, tensors)])
         except TypeError:  # not torch tensors: anything with a data_ptr()
             pass
-    return array.array("Q", [t.data_ptr() for t in tensors])
+    return array.array(N.WORD, [t.data_ptr() for t in tensors])
 
 
 class HostBuffer:
