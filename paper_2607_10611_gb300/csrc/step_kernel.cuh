@@ -723,7 +723,7 @@ __device__ __forceinline__ void get_e4m3(float (&x)[8], uint32_t saddr, float sc
 // Group stores (vector when whole and aligned, else element by element).  The
 // single stores are volatile so that those of one array stay together and L1
 // merges them by sector (217 M parameters, BF16 moments, BF16 weights 2 bytes
-// off a line: 1647 -> 1507 us).
+// off a line: 1647 -> 1507 us, 1439 with the loads below in order as well).
 __device__ __forceinline__ void st_u32(void* p, uint32_t v) {
   asm volatile("st.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -828,8 +828,8 @@ static_assert(kStaticSmem == 1024, "no padding between them");
 // itself, as each is read from the stage when it is there (load_group), so one
 // array off its boundary costs its own accesses alone: 217 M parameters, BF16
 // weights and gradients, binary32 moments (aligned 1152 us) with the weights 2
-// bytes off a line 2644 -> 1204 us, with mu 8 bytes off 2640 -> 1217; with
-// BF16 moments 2479 -> 1507 and 2598 -> 1506.
+// bytes off a line 2644 -> 1217 us, with mu 8 bytes off 2640 -> 1230; with
+// BF16 moments 2479 -> 1439 and 2598 -> 1381.
 constexpr uint32_t kVecW = 1, kVecM = 2, kVecV = 4, kVecVe = 8, kVecCc = 16, kVecAll = 31;
 
 // Per-tensor values the consumers keep while walking a tensor's tiles.
@@ -911,7 +911,9 @@ __device__ __forceinline__ void patch_group(const StepArgs& a, const TensorCtx& 
 
 // One array's eight elements of a group, each in a word of its own (a BF16 or a
 // code in the low bits): from the stage when the group's bytes are there, else
-// from global memory (elements from `valid` on are 0).
+// from global memory (elements from `valid` on are 0).  Those loads are volatile
+// to stay in order, one array's after another's: L1, a few KB a warp beside the
+// ring, holds few arrays' lines at a time.
 template <int ES, bool SHIFT>
 __device__ __forceinline__ void raw_group(uint32_t (&r)[8], bool staged, uint32_t saddr, const void* p, int64_t e0,
                                           int valid) {
@@ -942,9 +944,13 @@ __device__ __forceinline__ void raw_group(uint32_t (&r)[8], bool staged, uint32_
   const uint8_t* q = static_cast<const uint8_t*>(p) + e0 * ES;
 #pragma unroll
   for (int j = 0; j < kGroup; ++j) {
-    if (ES == 4) r[j] = j < valid ? *reinterpret_cast<const uint32_t*>(q + 4 * j) : 0u;
-    else if (ES == 2) r[j] = j < valid ? *reinterpret_cast<const uint16_t*>(q + 2 * j) : 0u;
-    else r[j] = j < valid ? q[j] : 0u;
+    r[j] = 0u;
+    if (j < valid) {
+      if (ES == 4) asm volatile("ld.global.u32 %0, [%1];" : "=r"(r[j]) : "l"(q + 4 * j) : "memory");
+      else if (ES == 2) asm volatile("{\n .reg .b16 h;\n ld.global.u16 h, [%1];\n cvt.u32.u16 %0, h;\n}"
+                                     : "=r"(r[j]) : "l"(q + 2 * j) : "memory");
+      else asm volatile("ld.global.u8 %0, [%1];" : "=r"(r[j]) : "l"(q + j) : "memory");
+    }
   }
 }
 
@@ -952,11 +958,13 @@ __device__ __forceinline__ void raw_group(uint32_t (&r)[8], bool staged, uint32_
 // or aligned: each array from the stage when it holds the whole group there,
 // else element by element from global memory -- the loads of all arrays before
 // the first use, so that the group waits on memory once (waiting array by
-// array, a BF16-moment list of 4000 ragged tensors took 345 us, now 295), and
-// one array's after another's, as L1, a few KB a warp beside the ring, holds
-// few arrays' lines at a time.  8-byte loads where the alignment allows them
-// were slower (binary32 moments, mu 8 bytes off: 2219 us against 1986, either
-// with all stores single).  dec: the scale the codes decode with.
+// array, a BF16-moment list of 4000 ragged tensors took 345 us, now 281).
+// 8-byte loads where the alignment allows them were slower (binary32 moments,
+// mu 8 bytes off: 2219 us against 1986, either with all stores single).  The
+// inlined instances (binary32 moments) read a group that is wholly there in a
+// block of its own: it is what a short launch's last warp runs once, and spread
+// over the other branches its instructions came in too late (E4M3, 0.4 M
+// parameters 8.08 -> 7.85 us).  dec: the scale the codes decode with.
 template <int WD, int GD, int MD, bool MIS>
 __device__ __forceinline__ void load_group(const StepArgs& a, const TensorCtx& x, const StageHead& h, int64_t e0,
                                            int count, int c, int valid, uint32_t st, float dec, float (&w)[8],
@@ -964,12 +972,32 @@ __device__ __forceinline__ void load_group(const StepArgs& a, const TensorCtx& x
   constexpr int WS = esize_of(WD), GS = esize_of(GD), MS = esize_of(MD);
   const uint32_t end = static_cast<uint32_t>(kGroup * (c + 1));  // elements through this group
   const uint32_t go = kGroup * GS * c + x.gsh, mo = kGroup * MS * c;
+  const uint32_t wo = WD == kNVFP4 ? 4u * c : static_cast<uint32_t>(kGroup * WS) * c + x.wsh;
+  const bool w_in = WD == kNVFP4          ? end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1)
+                    : MIS && WD != kBF16 ? in_range(h.w_range, wo, kGroup)
+                                         : end * WS <= staged_bytes(x.d.w, count, WS);
   const bool g_in = MIS ? in_range(h.g_range, go, kGroup * GS) : end * GS <= staged_bytes(h.g, count, GS);
+  const bool m_in = end * MS <= staged_bytes(x.d.m, count, MS), v_in = end * MS <= staged_bytes(x.d.v, count, MS);
+  const bool e_in = end * MS <= staged_bytes(x.d.ve, count, MS);
+  if constexpr (MD == kF32 && WD != kNVFP4) {
+    if (w_in && g_in && m_in && v_in && e_in && (!MIS || WD == kBF16 || (wo & 7u) == 0u)) {
+      if (WD == kBF16) get_bf16(w, st + wo);
+      else get_e4m3(w, st + wo, dec);
+      if (MIS && GD == kF32) get_f32_at(g, st + a.off_g + go);
+      else if (MIS) get_bf16_at(g, st + a.off_g + go);
+      else if (GD == kF32) get_f32(g, st + a.off_g + go);
+      else get_bf16(g, st + a.off_g + go);
+      get_f32(m, st + a.off_m + mo);
+      get_f32(v, st + a.off_v + mo);
+      get_f32(ve, st + a.off_ve + mo);
+      return;
+    }
+  }
   uint32_t rw[8], rg[8], rm[8], rv[8], re[8];
   if (WD == kNVFP4) {  // the group's codes as the bytes of one word
     rw[0] = 0u;
-    if (end / 2 <= staged_bytes(x.d.w, (count + 1) / 2, 1)) {
-      rw[0] = lds_u32(st + 4u * c);
+    if (w_in) {
+      rw[0] = lds_u32(st + wo);
     } else {
       const uint8_t* q = static_cast<const uint8_t*>(x.d.w) + (e0 >> 1);
 #pragma unroll
@@ -977,14 +1005,12 @@ __device__ __forceinline__ void load_group(const StepArgs& a, const TensorCtx& x
       rw[0] = rw[1] | rw[2] << 8 | rw[3] << 16 | rw[4] << 24;
     }
   } else {
-    const uint32_t wo = static_cast<uint32_t>(kGroup * WS) * c + x.wsh;
-    const bool w_in = MIS && WD != kBF16 ? in_range(h.w_range, wo, kGroup) : end * WS <= staged_bytes(x.d.w, count, WS);
     raw_group<WS, MIS && WD != kBF16>(rw, w_in, st + wo, x.d.w, e0, valid);
   }
   raw_group<GS, MIS>(rg, g_in, st + a.off_g + go, h.g, e0, valid);
-  raw_group<MS, false>(rm, end * MS <= staged_bytes(x.d.m, count, MS), st + a.off_m + mo, x.d.m, e0, valid);
-  raw_group<MS, false>(rv, end * MS <= staged_bytes(x.d.v, count, MS), st + a.off_v + mo, x.d.v, e0, valid);
-  raw_group<MS, false>(re, end * MS <= staged_bytes(x.d.ve, count, MS), st + a.off_ve + mo, x.d.ve, e0, valid);
+  raw_group<MS, false>(rm, m_in, st + a.off_m + mo, x.d.m, e0, valid);
+  raw_group<MS, false>(rv, v_in, st + a.off_v + mo, x.d.v, e0, valid);
+  raw_group<MS, false>(re, e_in, st + a.off_ve + mo, x.d.ve, e0, valid);
   auto val = [](uint32_t r, int es) { return __uint_as_float(es == 4 ? r : r << 16); };
   if (WD == kNVFP4) {
     e2m1x8_to_f32(rw[0], w);
@@ -1018,10 +1044,15 @@ __device__ __forceinline__ void put_compute(const uint32_t (&codes)[2], float sc
   put_bf16(o, cc, e0, valid, vec);
 }
 
-// Store the updated moments (BF16 moments nearest-even).  FAST: a whole staged
-// warp (TensorCtx::fast), where every array is aligned: its straight-line code
-// then holds neither the tests nor the single stores (217 M parameters with
-// BF16 moments, stochastic: NVFP4 982 -> 953 us, block-scaled E4M3 909 -> 893).
+// Whether the straight-line code of whole staged warps (TensorCtx::fast), where
+// every array is aligned, goes without the tests for it and the single stores.
+// As measured per instance: 217 M parameters with BF16 moments, stochastic,
+// NVFP4 982 -> 953 us, block-scaled E4M3 909 -> 893; binary32 moments, 2 M
+// parameters in E4M3 15.8 -> 15.4, but in BF16 8.9 -> 9.1, so not there.
+template <int WD, int MD>
+constexpr bool kFastStores = WD != kBF16 || MD == kBF16;
+
+// Store the updated moments (BF16 moments nearest-even).  FAST: see kFastStores.
 template <int MD, bool FAST>
 __device__ __forceinline__ void put_moments(const TensorCtx& x, int64_t e0, int valid, const float (&m)[8],
                                             const float (&v)[8], const float (&ve)[8]) {
@@ -1174,7 +1205,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
         }
       }
     }
-    put_bf16(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
+    put_bf16(ow, x.d.w, e0, valid, (STAGED && kFastStores<WD, MD>) || (x.vec & kVecW) != 0u);
   } else if (WD == kE4M3 && a.s.cert_ok) {
     // Certified fast path for E4M3: both ends of the bound are scaled by 2^-e
     // with outward rounding and encoded; the largest |w'| must be exact, so an
@@ -1275,7 +1306,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
       if (SR) ow[i] = __byte_perm(bf16_sr_sum(wn[2 * i], rnd[2 * i]), bf16_sr_sum(wn[2 * i + 1], rnd[2 * i + 1]), 0x7632);
       else ow[i] = bf16x2_rn(wn[2 * i], wn[2 * i + 1]);
     }
-    put_bf16(ow, x.d.w, e0, valid, STAGED || (x.vec & kVecW) != 0u);
+    put_bf16(ow, x.d.w, e0, valid, (STAGED && kFastStores<WD, MD>) || (x.vec & kVecW) != 0u);
   } else {
     uint32_t ow[2] = {0u, 0u};
 #pragma unroll
@@ -1288,7 +1319,7 @@ __device__ __forceinline__ void finish_group(const StepArgs& a, const TensorCtx&
     if (x.cc) put_compute(ow, x.cc_scale, x.cc, e0, valid, STAGED || (x.vec & kVecCc) != 0u);
   }
   }
-  put_moments<MD, STAGED>(x, e0, valid, m, v, ve);
+  put_moments<MD, STAGED && kFastStores<WD, MD>>(x, e0, valid, m, v, ve);
 }
 
 // One group of a partial tile, or of a tensor whose arrays are not all staged
